@@ -6,6 +6,7 @@
 
 #include "bcr.cuh"
 #include "tc_gemm.cuh"
+#include "tc_gemm64.cuh"
 
 namespace {
 
@@ -575,7 +576,8 @@ __device__ __forceinline__ bool gj_pivot(const cplx<T> (&x)[R], int k, int n, in
 template <typename T, bool SMEM, int R, int TR, int TC, int NT>
 __global__ void __launch_bounds__(NT)
 gj_regpanel_kernel(cplx<T>* __restrict__ src, int64_t src_stride, cplx<T>* __restrict__ out,
-                   int64_t out_stride, int n, int32_t* status) {
+                   int64_t out_stride, int n, int32_t* status, const int32_t* __restrict__ only) {
+  if (only && only[blockIdx.x] == 0) return;  // (only: the blocks to invert, null for all)
   constexpr int NB = NT / 32;
   constexpr int TY = NT / 32;
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -1006,14 +1008,15 @@ cudaError_t launch_gj_lookahead(const float2* src, int64_t src_stride, float2* o
 
 template <typename T, bool SMEM, int R, int TR, int TC, int NT>
 cudaError_t launch_gj_reg(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64_t out_stride,
-                          int n, int batch, int32_t* status, cudaStream_t s) {
+                          int n, int batch, int32_t* status, cudaStream_t s,
+                          const int32_t* only = nullptr) {
   const GjSmem<T> L(n, NT / 32, SMEM);
   if (L.total > SMEM_LIMIT || n > 32 * R) return cudaErrorInvalidValue;
   if (L.total > 48 * 1024)
     RCI_CUDA_TRY(cudaFuncSetAttribute(gj_regpanel_kernel<T, SMEM, R, TR, TC, NT>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
   gj_regpanel_kernel<T, SMEM, R, TR, TC, NT><<<batch, NT, L.total, s>>>(src, src_stride, out,
-                                                                        out_stride, n, status);
+                                                                        out_stride, n, status, only);
   rci_note_launch();
   return cudaGetLastError();
 }
@@ -1038,9 +1041,10 @@ cudaError_t launch_gj_cfg(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64_
 // global memory); larger blocks with gj_inverse_kernel.
 template <typename T>
 cudaError_t launch_gj_simt(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64_t out_stride,
-                           int n, int batch, int32_t* status, cudaStream_t s) {
+                           int n, int batch, int32_t* status, cudaStream_t s,
+                           const int32_t* only = nullptr) {
   if (batch <= 0) return cudaSuccess;
-  if (n > 1024) return cudaErrorInvalidValue;
+  if (n > 1024 || (only && (sizeof(T) == 4 || n > 256))) return cudaErrorInvalidValue;
   if constexpr (sizeof(T) == 4) {
     if (n <= 160 && GjLaSmem(n).total <= SMEM_LIMIT)
       return launch_gj_lookahead(src, src_stride, out, out_stride, n, batch, status, s);
@@ -1055,10 +1059,10 @@ cudaError_t launch_gj_simt(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64
   } else {
     if (n <= 160 && GjSmem<T>(n, 8, true).total <= SMEM_LIMIT)
       return launch_gj_reg<T, true, 5, 5, 5, 256>(src, src_stride, out, out_stride, n, batch,
-                                                  status, s);
+                                                  status, s, only);
     if (n <= 256)
       return launch_gj_reg<T, false, 8, 5, 5, 256>(src, src_stride, out, out_stride, n, batch,
-                                                   status, s);
+                                                   status, s, only);
     if (GjSmem<T>(n, 16, false).total <= SMEM_LIMIT)
       return launch_gj_cfg<T, false, 16, 5, 5, 256>(src, src_stride, out, out_stride, n, batch,
                                                     status, s);
@@ -1088,6 +1092,15 @@ __global__ void block_maxabs_kernel(const cplx<T>* __restrict__ a, int64_t strid
 }
 
 template <typename T>
+cudaError_t launch_block_maxabs(const cplx<T>* src, int64_t stride, int64_t nn, int batch, uint32_t* maxabs,
+                                cudaStream_t s) {
+  const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(nn * batch, 256), 4 * 152);
+  block_maxabs_kernel<T><<<grid, 256, 0, s>>>(src, stride, nn, batch, maxabs);
+  rci_note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
 cudaError_t launch_gj(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64_t out_stride, int n,
                       int batch, int32_t* status, cudaStream_t s, uint32_t* maxabs = nullptr,
                       bool tc = true) {
@@ -1096,14 +1109,8 @@ cudaError_t launch_gj(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64_t ou
     if (tc && n <= 160)
       return launch_tc_gj(src, src_stride, out, out_stride, n, batch, status, s, maxabs);
   }
-  if (maxabs) {
-    const int64_t nn = (int64_t)n * n;
-    const int64_t tot = nn * batch;
-    const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(tot, 256), 4 * 152);
-    block_maxabs_kernel<T><<<grid, 256, 0, s>>>(src, src_stride, nn, batch, maxabs);
-    rci_note_launch();
-    RCI_CUDA_TRY(cudaGetLastError());
-  }
+  if (maxabs)
+    RCI_CUDA_TRY(launch_block_maxabs<T>(src, src_stride, (int64_t)n * n, batch, maxabs, s));
   return launch_gj_simt<T>(src, src_stride, out, out_stride, n, batch, status, s);
 }
 
@@ -1997,6 +2004,267 @@ cudaError_t bcr_read_status(BcrHandle* h, int32_t* st, cudaStream_t s, double* g
   return cudaSuccess;
 }
 
+
+// ===================================================================== FP64 on the tensor cores
+// The FP64 factorisation runs its block products through the digit split of tc_gemm64.cu and its
+// block inverses as Newton iterations on an FP32 inverse, X <- X + X (I - D X), with those products:
+// the FP64 pipe does neither.  At ny = 160 a product takes 1.5 us of the whole GPU where the FP64
+// GEMM took 28, and an inverse of one block alone 0.4 ms where the FP64 Gauss-Jordan took 4.9: a
+// new design of 500 cells 404 -> 49 ms, of 50 cells (ny = 128) 54 -> 10.3 ms.
+// A block whose iteration does not contract (an FP32 inverse that resolves nothing, entries outside
+// the FP32 range, a singular block) goes to the FP64 Gauss-Jordan kernel, which also reports zero
+// pivots, so the factorisation accepts and refuses what it did.
+//
+// Scratch: the store of the level-0 inverses (G0), which no factorisation uses; the blocks of a
+// level are taken in batches that fit it.
+namespace {
+
+// a = (float) of `batch` nn-element blocks, stride elements apart
+__global__ void blocks_to_f32_kernel(const double2* __restrict__ src, int64_t stride, int64_t nn,
+                                     int64_t total, float2* __restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const int64_t z = e / nn;
+  const double2 v = src[z * stride + (e - z * nn)];
+  out[e] = make_float2((float)v.x, (float)v.y);
+}
+
+__global__ void blocks_to_f64_kernel(const float2* __restrict__ src, int64_t total,
+                                     double2* __restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < total) out[e] = make_double2((double)src[e].x, (double)src[e].y);
+}
+
+// After R = I - D X of one Newton step, per block (m = its largest |re|, |im|):
+// |R^2| <= 2 n m^2 bounds the residual that this step's update X + X R leaves.  When n m^2 is well
+// below rounding level the update is the last; an iteration that does not contract, or has not
+// got there at the last step, marks the block for the Gauss-Jordan kernel.  `rough`: R was
+// formed from the high digits only (SG_HALF), too coarse to end on.
+struct NewtonFlags {
+  uint32_t* maxabs;   // of R (bits of a float)
+  int32_t* skip_r;    // no further residual wanted
+  int32_t* skip_x;    // no further update wanted
+  int32_t* failed;
+};
+__global__ void newton_check_kernel(NewtonFlags f, int n, int batch, int rough, int last,
+                                    const int32_t* __restrict__ st32, int32_t* status) {
+  const int z = blockIdx.x * blockDim.x + threadIdx.x;
+  if (z == 0 && *st32 == DEV_TIMEOUT) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+  if (z >= batch) return;
+  if (f.skip_r[z]) {
+    f.skip_x[z] = 1;
+    return;
+  }
+  const float m = __uint_as_float(f.maxabs[z]);
+  f.maxabs[z] = 0;
+  const bool contracts = m * (float)n < 0.25f;
+  const bool done = contracts && !rough && (float)n * m * m <= 1e-17f;
+  if (!contracts || (last && !done)) f.failed[z] = f.skip_x[z] = 1;
+  if (!contracts || done || last) f.skip_r[z] = 1;
+}
+
+constexpr int NEWTON_STEPS = 4;
+
+// scratch of `bytes` at `base`, carved in 256-byte units
+struct Carve {
+  unsigned char* p;
+  template <typename P> P* take(size_t bytes) {
+    P* r = reinterpret_cast<P*>(p);
+    p += (bytes + 255) & ~(size_t)255;
+    return r;
+  }
+};
+inline size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
+
+// bytes per block of a batch: the Newton iteration, and the products of a reduction level
+size_t newton_block_bytes(int ny) {
+  const size_t nn = (size_t)ny * ny;
+  return 2 * up256(nn * 8) + up256(nn * 16) + 2 * sg_form_bytes(ny, ny, 3) + 2 * sg_form_bytes(ny, ny, 2) +
+         5 * 256 + 4 * up256(sizeof(int32_t) * sg_form_exps(ny));
+}
+size_t level_block_bytes(int ny) {
+  return 3 * sg_form_bytes(ny, ny, 3) + 2 * sg_form_bytes(ny, ny, 2) +
+         5 * up256(sizeof(int32_t) * sg_form_exps(ny));
+}
+
+}  // namespace
+
+// blocks per batch that `bytes` of scratch hold (0: the FP64 split path does not apply)
+static int split_batch(int ny, size_t bytes) {
+  if (ny > SG_KMAX) return 0;
+  const size_t per = std::max(newton_block_bytes(ny), level_block_bytes(ny));
+  const size_t fixed = 3 * level_block_bytes(ny) + 16 * 256;  // the levels' one extra block per form
+  return bytes <= fixed ? 0 : (int)std::min<size_t>((bytes - fixed) / per, 4096);
+}
+
+// out[z] = D[z]^-1 for z < m (D: stride elements apart, destroyed where the Gauss-Jordan kernel
+// takes over).
+static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int ny, int m, int cmax,
+                                 void* scratch, int32_t* status, cudaStream_t s) {
+  const int64_t nn = (int64_t)ny * ny;
+  const int nb = (int)ceil_div(m, cmax), cb = (int)ceil_div(m, nb);
+  const long long wl = tc_wait_limit();
+  for (int k0 = 0; k0 < m; k0 += cb) {
+    const int c = std::min(cb, m - k0);
+    Carve w{(unsigned char*)scratch};
+    float2* a32 = w.take<float2>((size_t)c * nn * 8);
+    float2* x32 = w.take<float2>((size_t)c * nn * 8);
+    double2* R = w.take<double2>((size_t)c * nn * 16);
+    const size_t f3 = sg_form_bytes(ny, ny, 3), f2 = sg_form_bytes(ny, ny, 2);
+    const int ne = sg_form_exps(ny);
+    unsigned char* fD = w.take<unsigned char>(c * f3);
+    unsigned char* fXr = w.take<unsigned char>(c * f3);
+    unsigned char* fXc = w.take<unsigned char>(c * f2);
+    unsigned char* fR = w.take<unsigned char>(c * f2);
+    int32_t* eD = w.take<int32_t>(sizeof(int32_t) * ne * c);
+    int32_t* eXr = w.take<int32_t>(sizeof(int32_t) * ne * c);
+    int32_t* eXc = w.take<int32_t>(sizeof(int32_t) * ne * c);
+    int32_t* eR = w.take<int32_t>(sizeof(int32_t) * ne * c);
+    int32_t* words = w.take<int32_t>(sizeof(int32_t) * (4 * (size_t)c + 1));
+    const NewtonFlags fl{reinterpret_cast<uint32_t*>(words), words + c, words + 2 * c, words + 3 * c};
+    int32_t* st32 = words + 4 * c;
+    double2* Dk = D + (int64_t)k0 * stride;
+    double2* X = out + (int64_t)k0 * nn;
+    RCI_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(int32_t) * (4 * (size_t)c + 1), s));
+    const int64_t tot = (int64_t)c * nn;
+    blocks_to_f32_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(Dk, stride, nn, tot, a32);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+    if (ny <= 160) RCI_CUDA_TRY(launch_tc_gj(a32, nn, x32, nn, ny, c, st32, s));
+    else RCI_CUDA_TRY(launch_gj_simt<float>(a32, nn, x32, nn, ny, c, st32, s));
+    blocks_to_f64_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(x32, tot, X);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+    RCI_CUDA_TRY(launch_sg_split(Dk, false, ny, stride, false, ny, ny, 3, c, fD, eD, nullptr, s));
+    for (int it = 0; it < NEWTON_STEPS; ++it) {
+      RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, true, ny, ny, 2, c, fXc, eXc, fl.skip_r, s));
+      SgJob r{};
+      r.nseg = 1;
+      r.seg[0] = SgSeg{fD, eD, fXc, eXc, 3, 2, 0, 0, 0, c};
+      r.neg = true;
+      r.identity = true;
+      r.C = R;
+      r.ldc = ny;
+      r.sC = nn;
+      r.batch = c;
+      r.maxabs = fl.maxabs;
+      r.skip = fl.skip_r;
+      RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &r, it == 0 ? SG_HALF : SG_FULL, status, wl, s));
+      newton_check_kernel<<<(unsigned)ceil_div(c, 128), 128, 0, s>>>(fl, ny, c, it == 0, it == NEWTON_STEPS - 1,
+                                                                     st32, status);
+      rci_note_launch();
+      RCI_CUDA_TRY(cudaGetLastError());
+      RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, false, ny, ny, 3, c, fXr, eXr, fl.skip_x, s));
+      RCI_CUDA_TRY(launch_sg_split(R, false, ny, nn, true, ny, ny, 2, c, fR, eR, fl.skip_x, s));
+      SgJob x{};
+      x.nseg = 1;
+      x.seg[0] = SgSeg{fXr, eXr, fR, eR, 3, 2, 0, 0, 0, c};
+      x.C0 = X;
+      x.ldc0 = ny;
+      x.sC0 = nn;
+      x.C = X;
+      x.ldc = ny;
+      x.sC = nn;
+      x.batch = c;
+      x.skip = fl.skip_x;
+      RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &x, SG_HALF, status, wl, s));
+    }
+    RCI_CUDA_TRY(launch_gj_simt<double>(Dk, stride, X, nn, ny, c, status, s, fl.failed));
+  }
+  return cudaSuccess;
+}
+
+// The products of one FP64 reduction level (the same five as the general path), in batches of
+// eliminated rows k0 .. k1 - 1:
+//   X_k = Dinv_k L_{2k+1};  Y_k = Dinv_k L_{2k+2}^T
+//   D'_k = D_{2k} - L_{2k} Y_{k-1} (k >= 1) - L_{2k+1}^T X_k (k < m);  L'_k = -L_{2k} X_{k-1} (k >= 1)
+// Every split form serves as often as it can: the columns of L_{2k+1} as the right operand of X
+// and the left one of D', the rows of L_{2k} as the right operand of Y (of the row before) and the
+// left one of D' and L'.
+static cudaError_t split_level(const double2* D, const double2* L, const double2* Dinv, double2* X, double2* Y,
+                               double2* Dn, double2* Ln, int ny, int n, int m, int nk, int cmax, void* scratch,
+                               int32_t* status, Profiler* prof, cudaStream_t s) {
+  const int64_t nn = (int64_t)ny * ny;
+  const int my = (n - 1) / 2;
+  const int nb = (int)ceil_div(nk, cmax), cb = (int)ceil_div(nk, nb);
+  const size_t f3 = sg_form_bytes(ny, ny, 3), f2 = sg_form_bytes(ny, ny, 2);
+  const int ne = sg_form_exps(ny);
+  const long long wl = tc_wait_limit();
+  for (int k0 = 0; k0 < nk; k0 += cb) {
+    const int c = std::min(cb, nk - k0);           // kept rows k0 .. k0 + c - 1
+    const int cm = std::min(c, m - k0);            // of which eliminated rows of the same index
+    const int cy = std::max(0, std::min(c, my - k0));
+    const int p0 = k0 > 0 ? 1 : 0;                 // X, Y of row k0 - 1 come first
+    Carve w{(unsigned char*)scratch};
+    unsigned char* fD = w.take<unsigned char>(c * f3);
+    unsigned char* fO = w.take<unsigned char>(c * f3);
+    unsigned char* fE = w.take<unsigned char>((c + 1) * f3);
+    unsigned char* fX = w.take<unsigned char>((c + 1) * f2);
+    unsigned char* fY = w.take<unsigned char>((c + 1) * f2);
+    int32_t* eD = w.take<int32_t>(sizeof(int32_t) * ne * c);
+    int32_t* eO = w.take<int32_t>(sizeof(int32_t) * ne * c);
+    int32_t* eE = w.take<int32_t>(sizeof(int32_t) * ne * (c + 1));
+    int32_t* eX = w.take<int32_t>(sizeof(int32_t) * ne * (c + 1));
+    int32_t* eY = w.take<int32_t>(sizeof(int32_t) * ne * (c + 1));
+    // L_{2k} for k = k0 .. k0 + c while it exists (index 2k <= n - 1; L_0 is not used)
+    const int nE = std::min(c + 1, nk - k0);
+    const int pm = p0 + std::max(0, cm), py = p0 + cy;
+    double flops = 8.0 * ny * (double)nn;
+    {
+      ProfScope ps(prof, PF_GEMM, s, flops * (std::max(0, cm) + cy), 3.0 * 16 * nn * (std::max(0, cm) + cy), 4);
+      if (cm > 0) {
+        RCI_CUDA_TRY(launch_sg_split(Dinv + k0 * nn, false, ny, nn, false, ny, ny, 3, cm, fD, eD, nullptr, s));
+        RCI_CUDA_TRY(launch_sg_split(L + (2 * (int64_t)k0 + 1) * nn, false, ny, 2 * nn, true, ny, ny, 3, cm, fO,
+                                     eO, nullptr, s));
+      }
+      // (k0 = 0: L_0 is uninitialised memory that no product reads; its form is skipped)
+      const int z0 = k0 == 0 ? 1 : 0;
+      if (nE > z0)
+        RCI_CUDA_TRY(launch_sg_split(L + 2 * (int64_t)(k0 + z0) * nn, false, ny, 2 * nn, false, ny, ny, 3, nE - z0,
+                                     fE + z0 * f3, eE + z0 * ne, nullptr, s));
+      SgJob xy[2] = {};
+      xy[0].nseg = 1;
+      xy[0].seg[0] = SgSeg{fD, eD, fO, eO, 3, 3, 0, 0, 0, std::max(0, cm)};
+      xy[0].C = X + k0 * nn;
+      xy[0].ldc = ny;
+      xy[0].sC = nn;
+      xy[0].batch = std::max(0, cm);
+      xy[1] = xy[0];
+      xy[1].seg[0] = SgSeg{fD, eD, fE, eE, 3, 3, 0, 1, 0, cy};
+      xy[1].C = Y + k0 * nn;
+      xy[1].batch = cy;
+      RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 2, xy, SG_FULL, status, wl, s));
+    }
+    ProfScope ps(prof, PF_GEMM, s, flops * (2.0 * (c - (k0 == 0)) + std::max(0, cm)), 16.0 * nn * 6 * c, 3);
+    if (pm > 0)
+      RCI_CUDA_TRY(launch_sg_split(X + (k0 - p0) * nn, false, ny, nn, true, ny, ny, 2, pm, fX, eX, nullptr, s));
+    if (py > 0)
+      RCI_CUDA_TRY(launch_sg_split(Y + (k0 - p0) * nn, false, ny, nn, true, ny, ny, 2, py, fY, eY, nullptr, s));
+    SgJob sl[2] = {};
+    const int lo = k0 == 0 ? 1 : 0;                // row 0 has no row before it
+    sl[0].nseg = 2;
+    sl[0].seg[0] = SgSeg{fE, eE, fY, eY, 3, 2, 0, p0 - 1, lo, c};
+    sl[0].seg[1] = SgSeg{fO, eO, fX, eX, 3, 2, 0, p0, 0, std::max(0, cm)};
+    sl[0].neg = true;
+    sl[0].C0 = D + 2 * (int64_t)k0 * nn;
+    sl[0].ldc0 = ny;
+    sl[0].sC0 = 2 * nn;
+    sl[0].C = Dn + k0 * nn;
+    sl[0].ldc = ny;
+    sl[0].sC = nn;
+    sl[0].batch = c;
+    sl[1].nseg = 1;
+    sl[1].seg[0] = SgSeg{fE + lo * f3, eE + lo * ne, fX, eX, 3, 2, 0, p0 - 1 + lo, 0, c - lo};
+    sl[1].neg = true;
+    sl[1].C = Ln + (k0 + lo) * nn;
+    sl[1].ldc = ny;
+    sl[1].sC = nn;
+    sl[1].batch = c - lo;
+    RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 2, sl, SG_FULL, status, wl, s));
+  }
+  return cudaSuccess;
+}
+
 template <typename T>
 static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, const double2* cy,
                             cudaStream_t s) {
@@ -2050,6 +2318,10 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
   const cplx<T> one = mkc(T(1), T(0)), mone = mkc(T(-1), T(0)), zero = czero<T>();
   int cur = 0;
   auto store = (cplx<T>*)h->store;
+  // FP64 on the tensor cores where the scratch holds at least one block
+  int cmax = 0;
+  if constexpr (sizeof(T) == 8)
+    cmax = split_batch(ny, (size_t)std::max<int64_t>(m0, 1) * nn * sizeof(cplx<T>));
   for (int l = 1; l < h->Lf; ++l) {
     const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
     const int my = (n - 1) / 2;
@@ -2063,7 +2335,13 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     // D_r^{-1} for the odd rows (the working copy of D_r is destroyed)
     {
       ProfScope ps(h->prof, PF_INVERT, s, 8.0 * ny * (double)nn * m, 2.0 * m * nn * sizeof(cplx<T>), 1);
-      RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
+      if constexpr (sizeof(T) == 8) {
+        if (cmax > 0) {
+          RCI_CUDA_TRY(launch_block_maxabs<T>(D + nn, 2 * nn, nn, m, maxabs + 1, s));
+          RCI_CUDA_TRY(split_inverse(D + nn, 2 * nn, Dinv, ny, m, cmax, h->G0, h->status, s));
+        }
+      }
+      if (cmax == 0) RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
                                 !h->simt));
     }
     // X_k = Dinv_k L_{2k+1};  Y_k = Dinv_k L_{2k+2}^T
@@ -2072,6 +2350,12 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     // FP32 on the tensor cores: two launches, X and Y together, then each D' as one product
     // over K = 2 ny (written once) together with L'; otherwise five batched products.
     bool fused = false;
+    if constexpr (sizeof(T) == 8) {
+      if (cmax > 0) {
+        RCI_CUDA_TRY(split_level(D, L, Dinv, X, Y, Dn, Ln, ny, n, m, nk, cmax, h->G0, h->status, h->prof, s));
+        fused = true;
+      }
+    }
     if constexpr (sizeof(T) == 4) {
       if (nk >= 2 && my >= 1) {
         const double pb = (double)sizeof(cplx<T>) * nn;
@@ -2142,6 +2426,12 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
   // last single row
   {
     ProfScope ps(h->prof, PF_INVERT, s, 8.0 * ny * (double)nn, 2.0 * nn * sizeof(cplx<T>), 1);
+    if constexpr (sizeof(T) == 8) {
+      if (cmax > 0) {
+        RCI_CUDA_TRY(launch_block_maxabs<T>((cplx<T>*)h->Dw[cur], nn, nn, 1, maxabs + 1, s));
+        return split_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, cmax, h->G0, h->status, s);
+      }
+    }
     RCI_CUDA_TRY(launch_gj<T>((cplx<T>*)h->Dw[cur], 0, store + h->final_off, 0, ny, 1, h->status, s,
                               maxabs + 1, !h->simt));
   }

@@ -419,6 +419,7 @@ rci_status fp64_fallback(rci_grid* g) {
   CK(bcr_factor(g->bcr64, g->dg, g->cx, g->cy, g->s), "FP64 fallback factor");
   int32_t st = 0;
   CK(bcr_read_status(g->bcr64, &st, g->s, &g->growth64), "FP64 fallback status");
+  if (st == DEV_TIMEOUT) return fail(g, RCI_ETIMEOUT, "a bounded tensor-core wait expired");
   if (st == DEV_SINGULAR) return fail(g, RCI_ESINGULAR, "zero pivot in a diagonal block (FP64)");
   g->use64 = true;
   return RCI_OK;
