@@ -45,6 +45,7 @@ struct rci_grid {
   double* part_b = nullptr;
   double* ratio = nullptr;  // per-RHS residual ratio (up to MAXQ)
   double* vf_scratch = nullptr;
+  bool vf_rule = false;  // vf_scratch holds the Gauss-Legendre rule (the same for every objective)
   int32_t* dstatus = nullptr;
   // multi right-hand side buffers (grown on demand)
   int mq_cap = 0;
@@ -318,8 +319,10 @@ rci_status build_objective(rci_grid* g, const rci_objective* o, double2* b) {
     CK(launch_planewave_row(G, o->theta_out, g->crow, g->s), "planewave objective");
   } else if (o->kind == RCI_OBJ_VIRTUAL_FOCUS) {
     if (o->d_rows < 0) return fail(g, RCI_EINVAL, "d_rows must be >= 0");
-    CK(launch_virtual_focus_row(G, o->x_f, o->d_rows, g->crow, g->vf_scratch, g->s),
+    // r1 (N complex) is free until the solve: the partial sums of the node chunks
+    CK(launch_virtual_focus_row(G, o->x_f, o->d_rows, g->crow, g->vf_scratch, g->vf_rule, g->r1, g->s),
        "virtual focus objective");
+    g->vf_rule = true;
   } else if (o->kind == RCI_OBJ_USER_ROW) {
     if (!o->w_row) return fail(g, RCI_EINVAL, "w_row is NULL");
     CK(cudaMemcpyAsync(g->crow, o->w_row, sizeof(double2) * G.n_src, cudaMemcpyHostToDevice, g->s),
