@@ -168,18 +168,14 @@ __device__ __forceinline__ void tri_forward_unit(const TriRow<T>& f, int n, int 
 // b - 1 on, the others being zero), then one backward sweep runs both recurrences side by
 // side, so that every entry of D'_k is formed in one step (no read-back of a partial D'),
 // with the scratch loads issued a few rows ahead.
-// MODE 1 forms instead the dense T_{2k+1}^{-1} of the eliminated rows k < m0 (the stored
-// inverses of the solve with several right-hand sides), one block each, the forward sweep
-// written in place into the output column: the backward sweep reads row a - PF before it
-// writes row a, so every row is read before it is overwritten.
-template <typename T, int MODE>
+template <typename T>
 __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double2* __restrict__ cx,
                                     const double2* __restrict__ cy, int nx, int ny,
                                     const cplx<T>* __restrict__ tdl, const cplx<T>* __restrict__ tdinv,
                                     const cplx<T>* __restrict__ tdu, const cplx<T>* __restrict__ tdu2,
                                     const uint8_t* __restrict__ tpiv, cplx<T>* __restrict__ Dn,
-                                    cplx<T>* __restrict__ Ln, cplx<T>* scrR,
-                                    cplx<T>* __restrict__ scrL, cplx<T>* G0) {
+                                    cplx<T>* __restrict__ Ln, cplx<T>* __restrict__ scrR,
+                                    cplx<T>* __restrict__ scrL) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   cplx<T>* sm = reinterpret_cast<cplx<T>*>(sm_raw);
   // [0,4ny): right factors, [4ny,8ny): left factors, then cxl2, cxl, cxr, dge, cye; piv bytes last
@@ -195,8 +191,8 @@ __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double
 
   const int k = blockIdx.x;
   const int64_t e = 2 * (int64_t)k;
-  const bool has_r = MODE == 1 || e + 1 < nx;   // eliminated row e+1 has index k
-  const bool has_l = MODE == 0 && e >= 1;       // eliminated row e-1 has index k-1
+  const bool has_r = e + 1 < nx;   // eliminated row e+1 has index k
+  const bool has_l = e >= 1;       // eliminated row e-1 has index k-1
   for (int j = threadIdx.x; j < ny; j += blockDim.x) {
     if (has_r) {
       int64_t b = (int64_t)k * ny + j;
@@ -206,7 +202,6 @@ __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double
       R[3 * ny + j] = tdu2[b];
       pivR[j] = tpiv[b];
     }
-    if (MODE == 1) continue;
     cxr[j] = has_r ? ccast<T>(cx[e * ny + j]) : czero<T>();
     if (has_l) {
       int64_t b = (int64_t)(k - 1) * ny + j;
@@ -229,18 +224,14 @@ __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double
   const int64_t nn = (int64_t)ny * ny;
   cplx<T>* __restrict__ Dcol = Dn + (int64_t)k * nn + b;
   cplx<T>* __restrict__ Lcol = Ln + (int64_t)k * nn + b;
-  cplx<T>* Gcol = G0 + (int64_t)k * nn + b;
-  // MODE 1: the sweep in place in the output column
-  cplx<T>* YR = MODE == 1 ? Gcol : scrR + (int64_t)k * nn + b;
+  cplx<T>* __restrict__ YR = scrR + (int64_t)k * nn + b;
   cplx<T>* __restrict__ YL = scrL + (int64_t)k * nn + b;
   const TriRow<T> fR{R, R + ny, R + 2 * ny, R + 3 * ny, pivR};
   const TriRow<T> fL{Lf, Lf + ny, Lf + 2 * ny, Lf + 3 * ny, pivL};
   if (has_r) tri_forward_unit<T>(fR, ny, b, YR, ny);
   if (has_l) tri_forward_unit<T>(fL, ny, b, YL, ny);
   const int a_lo = b > 0 ? b - 1 : 0;  // first row the sweeps wrote
-  const cplx<T> sb = MODE == 0 ? cxr[b] : czero<T>();
-  const cplx<T> sl = MODE == 0 ? cxl[b] : czero<T>();
-  const cplx<T> sl2 = MODE == 0 ? cxl2[b] : czero<T>();
+  const cplx<T> sb = cxr[b], sl = cxl[b], sl2 = cxl2[b];
   cplx<T> r1 = czero<T>(), r2 = czero<T>(), l1 = czero<T>(), l2 = czero<T>();
   // scratch values of the next PF rows, loaded ahead of the recurrences
   constexpr int PF = 4;
@@ -265,10 +256,6 @@ __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double
       if (!has_r) gr = czero<T>();
       r2 = r1;
       r1 = gr;
-      if (MODE == 1) {
-        Gcol[(int64_t)a * ny] = gr;
-        continue;
-      }
       cplx<T> gl = cfms(fL.du2[a], l2, cfms(fL.du[a], l1, cl)) * fL.dinv[a];
       if (!has_l) gl = czero<T>();
       l2 = l1;
@@ -1292,96 +1279,120 @@ cudaError_t gemm(int M, int N, int K, bool ta, bool tb, cplx<T> alpha, const cpl
 }
 
 // ===================================================================== solve kernels
-// Level 0 forward: t0[k] = T_{2k+1}^{-1} b[2k+1] (one thread per (k, q)).
-template <typename T>
-__global__ void fwd0_kernel(const cplx<T>* __restrict__ b, cplx<T>* __restrict__ t0, int ny,
-                            int m0, int nrhs, const cplx<T>* tdl, const cplx<T>* tdinv,
-                            const cplx<T>* tdu, const cplx<T>* tdu2, const uint8_t* tpiv) {
-  int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tt >= (int64_t)m0 * nrhs) return;
-  int k = (int)(tt / nrhs), q = (int)(tt - (int64_t)k * nrhs);
-  int64_t fb = (int64_t)k * ny;
-  TriRow<T> f{tdl + fb, tdinv + fb, tdu + fb, tdu2 + fb, tpiv + fb};
-  const cplx<T>* br = b + (2 * (int64_t)k + 1) * ny * nrhs + q;
-  cplx<T>* tr = t0 + (int64_t)k * ny * nrhs + q;
-  tri_forward<T>(f, ny, [&](int j) { return br[(int64_t)j * nrhs]; },
-                 [&](int j, cplx<T> y) { tr[(int64_t)j * nrhs] = y; });
-  tri_backward<T>(f, ny, [&](int j) { return tr[(int64_t)j * nrhs]; },
-                  [&](int j, cplx<T> g) { tr[(int64_t)j * nrhs] = g; });
+// Sweeps with the tridiagonal factors for one right-hand side per thread, TRM_PF rows at a time:
+// their right-hand sides and factors are loaded before the recurrence runs over them, so that a
+// thread waits for memory once per TRM_PF rows.  out rows are ld apart.
+constexpr int TRM_PF = 8;
+
+template <typename T, typename Rhs>
+__device__ __forceinline__ void tri_solve_rows(const TriRow<T>& f, int n, Rhs rhs, cplx<T>* out, int64_t ld) {
+  cplx<T> cur = rhs(0);
+  for (int j0 = 0; j0 < n - 1; j0 += TRM_PF) {
+    cplx<T> nb[TRM_PF], l[TRM_PF];
+    bool pv[TRM_PF];
+#pragma unroll
+    for (int q = 0; q < TRM_PF; ++q) {
+      const int j = j0 + q < n - 1 ? j0 + q : n - 2;
+      nb[q] = rhs(j + 1);
+      l[q] = f.dl[j];
+      pv[q] = f.piv[j] != 0;
+    }
+#pragma unroll
+    for (int q = 0; q < TRM_PF; ++q) {
+      if (j0 + q >= n - 1) break;
+      out[(j0 + q) * ld] = pv[q] ? nb[q] : cur;
+      cur = pv[q] ? cfms(l[q], nb[q], cur) : cfms(l[q], cur, nb[q]);
+    }
+  }
+  out[(n - 1) * ld] = cur;
+  cplx<T> g1 = czero<T>(), g2 = czero<T>();  // g_{j+1}, g_{j+2}
+  for (int j0 = n - 1; j0 >= 0; j0 -= TRM_PF) {
+    cplx<T> y[TRM_PF], du[TRM_PF], du2[TRM_PF], di[TRM_PF];
+#pragma unroll
+    for (int q = 0; q < TRM_PF; ++q) {
+      const int j = j0 - q > 0 ? j0 - q : 0;
+      y[q] = out[j * ld];
+      du[q] = f.du[j];
+      du2[q] = f.du2[j];
+      di[q] = f.dinv[j];
+    }
+#pragma unroll
+    for (int q = 0; q < TRM_PF; ++q) {
+      if (j0 - q < 0) break;
+      const cplx<T> g = cfms(du2[q], g2, cfms(du[q], g1, y[q])) * di[q];
+      out[(j0 - q) * ld] = g;
+      g2 = g1;
+      g1 = g;
+    }
+  }
 }
 
-// Level 0 kept rows: B1[k] = b[2k] - cx[2k-1] o t0[k-1] - cx[2k] o t0[k].
+// Level 0 forward: t0[k] = T_{2k+1}^{-1} b[2k+1] (one thread per (k, q)).  b: nrhs columns, t0:
+// ld >= nrhs columns.
+template <typename T>
+__global__ void __launch_bounds__(128)
+fwd0_kernel(const cplx<T>* __restrict__ b, cplx<T>* __restrict__ t0, int ny, int m0, int nrhs, int ld,
+            const cplx<T>* __restrict__ tdl, const cplx<T>* __restrict__ tdinv, const cplx<T>* __restrict__ tdu,
+            const cplx<T>* __restrict__ tdu2, const uint8_t* __restrict__ tpiv) {
+  const int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tt >= (int64_t)m0 * nrhs) return;
+  const int k = (int)(tt / nrhs), q = (int)(tt - (int64_t)k * nrhs);
+  const int64_t fb = (int64_t)k * ny;
+  const TriRow<T> f{tdl + fb, tdinv + fb, tdu + fb, tdu2 + fb, tpiv + fb};
+  const cplx<T>* br = b + (2 * (int64_t)k + 1) * ny * nrhs + q;
+  tri_solve_rows<T>(f, ny, [&](int j) { return br[(int64_t)j * nrhs]; }, t0 + (int64_t)k * ny * ld + q, ld);
+}
+
+// Level 0 kept rows: B1[k] = b[2k] - cx[2k-1] o t0[k-1] - cx[2k] o t0[k].  b: nrhs columns, t0 and
+// B1: ld (the columns from nrhs on are zero).
 template <typename T>
 __global__ void keep0_kernel(const cplx<T>* __restrict__ b, const cplx<T>* __restrict__ t0,
                              const double2* __restrict__ cx, cplx<T>* __restrict__ B1, int nx,
-                             int ny, int n1, int nrhs) {
-  int64_t row = (int64_t)ny * nrhs;
-  int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+                             int ny, int n1, int nrhs, int ld) {
+  const int64_t row = (int64_t)ny * ld;
+  const int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (tt >= (int64_t)n1 * row) return;
-  int64_t k = tt / row, r = tt - k * row;
-  int j = (int)(r / nrhs);
-  cplx<T> v = b[2 * k * row + r];
-  if (k >= 1) v = cfms(ccast<T>(cx[(2 * k - 1) * ny + j]), t0[(k - 1) * row + r], v);
-  if (2 * k + 1 < nx) v = cfms(ccast<T>(cx[(2 * k) * ny + j]), t0[k * row + r], v);
+  const int64_t k = tt / row, r = tt - k * row;
+  const int j = (int)(r / ld), q = (int)(r - (int64_t)j * ld);
+  cplx<T> v = czero<T>();
+  if (q < nrhs) {
+    v = b[(2 * k * ny + j) * nrhs + q];
+    if (k >= 1) v = cfms(ccast<T>(cx[(2 * k - 1) * ny + j]), t0[(k - 1) * row + r], v);
+    if (2 * k + 1 < nx) v = cfms(ccast<T>(cx[(2 * k) * ny + j]), t0[k * row + r], v);
+  }
   B1[tt] = v;
 }
 
 // Level 0 back substitution: x[2k] = x1[k];
-// x[2k+1] = T^{-1}(b[2k+1] - cx[2k] o x1[k] - cx[2k+1] o x1[k+1]).
+// x[2k+1] = T^{-1}(b[2k+1] - cx[2k] o x1[k] - cx[2k+1] o x1[k+1]).  x1: ld columns.
 template <typename T>
-__global__ void bwd0_kernel(const cplx<T>* b, const cplx<T>* __restrict__ x1,
-                            const double2* __restrict__ cx, cplx<T>* x, int nx, int ny, int n1,
-                            int nrhs, const cplx<T>* tdl, const cplx<T>* tdinv, const cplx<T>* tdu,
-                            const cplx<T>* tdu2, const uint8_t* tpiv) {
-  int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128)
+bwd0_kernel(const cplx<T>* __restrict__ b, const cplx<T>* __restrict__ x1, const double2* __restrict__ cx,
+            cplx<T>* __restrict__ x, int nx, int ny, int n1, int nrhs, int ld, const cplx<T>* __restrict__ tdl,
+            const cplx<T>* __restrict__ tdinv, const cplx<T>* __restrict__ tdu, const cplx<T>* __restrict__ tdu2,
+            const uint8_t* __restrict__ tpiv) {
+  const int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (tt >= (int64_t)n1 * nrhs) return;
-  int k = (int)(tt / nrhs), q = (int)(tt - (int64_t)k * nrhs);
-  int64_t row = (int64_t)ny * nrhs;
-  const cplx<T>* xa = x1 + (int64_t)k * row + q;
+  const int k = (int)(tt / nrhs), q = (int)(tt - (int64_t)k * nrhs);
+  const int64_t row = (int64_t)ny * nrhs, row1 = (int64_t)ny * ld;
+  const cplx<T>* xa = x1 + (int64_t)k * row1 + q;
   cplx<T>* xe = x + 2 * (int64_t)k * row + q;
-  for (int j = 0; j < ny; ++j) xe[(int64_t)j * nrhs] = xa[(int64_t)j * nrhs];
-  int64_t r = 2 * (int64_t)k + 1;
+#pragma unroll 8
+  for (int j = 0; j < ny; ++j) xe[(int64_t)j * nrhs] = xa[(int64_t)j * ld];
+  const int64_t r = 2 * (int64_t)k + 1;
   if (r >= nx) return;
   const bool has_b = r + 1 < nx;
-  const cplx<T>* xb = x1 + (int64_t)(k + 1) * row + q;
+  const cplx<T>* xb = has_b ? xa + row1 : xa;
   const cplx<T>* br = b + r * row + q;
-  cplx<T>* xr = x + r * row + q;
   const double2* cl = cx + (r - 1) * ny;
   const double2* cr = cx + r * ny;
-  int64_t fb = (int64_t)k * ny;
-  TriRow<T> f{tdl + fb, tdinv + fb, tdu + fb, tdu2 + fb, tpiv + fb};
-  auto rhs = [&](int j) {
-    cplx<T> v = cfms(ccast<T>(cl[j]), xa[(int64_t)j * nrhs], br[(int64_t)j * nrhs]);
-    if (has_b) v = cfms(ccast<T>(cr[j]), xb[(int64_t)j * nrhs], v);
-    return v;
-  };
-  tri_forward<T>(f, ny, rhs, [&](int j, cplx<T> y) { xr[(int64_t)j * nrhs] = y; });
-  tri_backward<T>(f, ny, [&](int j) { return xr[(int64_t)j * nrhs]; },
-                  [&](int j, cplx<T> g) { xr[(int64_t)j * nrhs] = g; });
-}
-
-// Kept rows of a dense level: Bn[k] = B[2k] - Q[k-1] - P[k].
-template <typename T>
-__global__ void keep_kernel(const cplx<T>* __restrict__ B, const cplx<T>* __restrict__ P,
-                            const cplx<T>* __restrict__ Q, cplx<T>* __restrict__ Bn, int m, int nk,
-                            int64_t row) {
-  int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tt >= (int64_t)nk * row) return;
-  int64_t k = tt / row, r = tt - k * row;
-  cplx<T> v = B[2 * k * row + r];
-  if (k >= 1) v = v - Q[(k - 1) * row + r];
-  if (k < m) v = v - P[k * row + r];
-  Bn[tt] = v;
-}
-
-// x_l[2k] = x_up[k] for every kept row.
-template <typename T>
-__global__ void copy_kept_kernel(const cplx<T>* __restrict__ xup, cplx<T>* __restrict__ xl, int nk,
-                                 int64_t row) {
-  int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tt >= (int64_t)nk * row) return;
-  int64_t k = tt / row, r = tt - k * row;
-  xl[2 * k * row + r] = xup[tt];
+  const int64_t fb = (int64_t)k * ny;
+  const TriRow<T> f{tdl + fb, tdinv + fb, tdu + fb, tdu2 + fb, tpiv + fb};
+  tri_solve_rows<T>(f, ny, [&](int j) {
+    cplx<T> v = cfms(ccast<T>(cl[j]), xa[(int64_t)j * ld], br[(int64_t)j * nrhs]);
+    const cplx<T> c = has_b ? ccast<T>(cr[j]) : czero<T>();
+    return has_b ? cfms(c, xb[(int64_t)j * ld], v) : v;
+  }, x + r * row + q, nrhs);
 }
 
 // sum of a complex value over the 32 lanes of a warp (every lane gets the sum)
@@ -1392,27 +1403,6 @@ __device__ __forceinline__ cplx<T> warp_sum(cplx<T> v) {
     v.y += __shfl_xor_sync(0xffffffffu, v.y, off);
   }
   return v;
-}
-
-// Level 0 backward, several right-hand sides: x[2k] = x1[k] and the right-hand sides of
-// the eliminated rows, tmp[k] = b[2k+1] - cx[2k] o x1[k] - cx[2k+1] o x1[k+1].
-template <typename T>
-__global__ void bwd0_rhs_kernel(const cplx<T>* b, const cplx<T>* __restrict__ x1,
-                                const double2* __restrict__ cx, cplx<T>* x,
-                                cplx<T>* __restrict__ tmp, int nx, int ny, int n1, int nrhs) {
-  const int64_t row = (int64_t)ny * nrhs;
-  const int64_t tt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tt >= (int64_t)n1 * row) return;
-  const int64_t k = tt / row, e = tt - k * row;
-  const int j = (int)(e / nrhs);
-  const int64_t r = 2 * k + 1;
-  const cplx<T> xa = x1[tt];
-  if (r < nx) {
-    cplx<T> v = cfms(ccast<T>(cx[(r - 1) * ny + j]), xa, b[r * row + e]);
-    if (r + 1 < nx) v = cfms(ccast<T>(cx[r * ny + j]), x1[(k + 1) * row + e], v);
-    tmp[k * row + e] = v;
-  }
-  x[2 * k * row + e] = xa;
 }
 
 // ----- single right-hand side, chunked: a block per (block row k, chunk of RC rows or
@@ -1888,8 +1878,7 @@ struct BcrHandle {
   // factor storage
   void *tdl = nullptr, *tdinv = nullptr, *tdu = nullptr, *tdu2 = nullptr;
   uint8_t* tpiv = nullptr;
-  void* G0 = nullptr;             // dense T_r^{-1} of the level-0 eliminated rows (m0 x ny x ny)
-  bool g0_valid = false;          // G0 holds the inverses of the current factorisation
+  void* scratch = nullptr;        // m0 x ny x ny elements: the FP64 split path's digits and blocks
   bool simt = false;              // FP32: factor and multi-RHS products on the SIMT pipe
   void* Dw[2] = {nullptr, nullptr};
   void* Lw[2] = {nullptr, nullptr};
@@ -1913,7 +1902,7 @@ static void free_ws(BcrHandle* h) {
 
 void bcr_destroy(BcrHandle* h) {
   if (!h) return;
-  void* ps[] = {h->tdl, h->tdinv, h->tdu, h->tdu2, h->tpiv, h->G0, h->Dw[0], h->Dw[1],
+  void* ps[] = {h->tdl, h->tdinv, h->tdu, h->tdu2, h->tpiv, h->scratch, h->Dw[0], h->Dw[1],
                 h->Lw[0], h->Lw[1], h->store, h->status};
   for (void* p : ps) h->mem.release(p);
   free_ws(h);
@@ -1974,7 +1963,7 @@ cudaError_t bcr_create(int nx, int ny, int prec, const DevMem* mem, BcrHandle** 
   alloc(&h->tdu, m0b * h->esz);
   alloc(&h->tdu2, m0b * h->esz);
   alloc((void**)&h->tpiv, m0b);
-  alloc(&h->G0, m0b * ny * h->esz);
+  alloc(&h->scratch, m0b * ny * h->esz);
   for (int i = 0; i < 2; ++i) {
     alloc(&h->Dw[i], (size_t)n1 * nn * h->esz);
     alloc(&h->Lw[i], (size_t)n1 * nn * h->esz);
@@ -2015,8 +2004,8 @@ cudaError_t bcr_read_status(BcrHandle* h, int32_t* st, cudaStream_t s, double* g
 // the FP32 range, a singular block) goes to the FP64 Gauss-Jordan kernel, which also reports zero
 // pivots, so the factorisation accepts and refuses what it did.
 //
-// Scratch: the store of the level-0 inverses (G0), which no factorisation uses; the blocks of a
-// level are taken in batches that fit it.
+// Scratch: the handle's (m0 blocks of ny x ny); the blocks of a level are taken in batches that
+// fit it.
 namespace {
 
 // a = (float) of `batch` nn-element blocks, stride elements apart
@@ -2298,21 +2287,18 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     RCI_CUDA_TRY(cudaGetLastError());
   }
   {
-    // D' and L' of the first reduced system; the stored inverses G0 are formed when a solve
-    // with several right-hand sides first needs them
+    // D' and L' of the first reduced system
     const int thr = (int)ceil_div(ny, 32) * 32;
     const size_t smem = l0_smem<T>(ny);
     if (smem > 48 * 1024)
-      RCI_CUDA_TRY(cudaFuncSetAttribute(level0_schur_kernel<T, 0>,
+      RCI_CUDA_TRY(cudaFuncSetAttribute(level0_schur_kernel<T>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // the next level's working arrays are free during level 0 and serve as scratch
-    level0_schur_kernel<T, 0><<<n1, thr, smem, s>>>(dg, cx, cy, nx, ny, tdl, tdinv, tdu, tdu2,
+    level0_schur_kernel<T><<<n1, thr, smem, s>>>(dg, cx, cy, nx, ny, tdl, tdinv, tdu, tdu2,
                                                     h->tpiv, (cplx<T>*)h->Dw[0], (cplx<T>*)h->Lw[0],
-                                                    (cplx<T>*)h->Dw[1], (cplx<T>*)h->Lw[1],
-                                                    (cplx<T>*)h->G0);
+                                                    (cplx<T>*)h->Dw[1], (cplx<T>*)h->Lw[1]);
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
-    h->g0_valid = false;
   }
   delete l0;
   const cplx<T> one = mkc(T(1), T(0)), mone = mkc(T(-1), T(0)), zero = czero<T>();
@@ -2338,7 +2324,7 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
       if constexpr (sizeof(T) == 8) {
         if (cmax > 0) {
           RCI_CUDA_TRY(launch_block_maxabs<T>(D + nn, 2 * nn, nn, m, maxabs + 1, s));
-          RCI_CUDA_TRY(split_inverse(D + nn, 2 * nn, Dinv, ny, m, cmax, h->G0, h->status, s));
+          RCI_CUDA_TRY(split_inverse(D + nn, 2 * nn, Dinv, ny, m, cmax, h->scratch, h->status, s));
         }
       }
       if (cmax == 0) RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
@@ -2352,7 +2338,7 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     bool fused = false;
     if constexpr (sizeof(T) == 8) {
       if (cmax > 0) {
-        RCI_CUDA_TRY(split_level(D, L, Dinv, X, Y, Dn, Ln, ny, n, m, nk, cmax, h->G0, h->status, h->prof, s));
+        RCI_CUDA_TRY(split_level(D, L, Dinv, X, Y, Dn, Ln, ny, n, m, nk, cmax, h->scratch, h->status, h->prof, s));
         fused = true;
       }
     }
@@ -2429,7 +2415,7 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     if constexpr (sizeof(T) == 8) {
       if (cmax > 0) {
         RCI_CUDA_TRY(launch_block_maxabs<T>((cplx<T>*)h->Dw[cur], nn, nn, 1, maxabs + 1, s));
-        return split_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, cmax, h->G0, h->status, s);
+        return split_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, cmax, h->scratch, h->status, s);
       }
     }
     RCI_CUDA_TRY(launch_gj<T>((cplx<T>*)h->Dw[cur], 0, store + h->final_off, 0, ny, 1, h->status, s,
@@ -2444,16 +2430,22 @@ cudaError_t bcr_factor(BcrHandle* h, const double2* dg, const double2* cx, const
                              : factor_t<float>(h, dg, cx, cy, s);
 }
 
-// workspace layout for nrhs right-hand sides (elements of cplx<T>):
-//   t0 [m0 row] | B_l [n_l row] (l = 1..Lf) | t_l [m_l row] (l = 1..Lf-1) | P, Q [m_1 row] | xf [row]
+// columns of the workspace rows for nrhs right-hand sides (even in FP32: the TMA-fed products take
+// 16-byte aligned rows)
+static int ws_cols(const BcrHandle* h, int nrhs) { return h->prec == RCI_FP64 ? nrhs : (nrhs + 1) & ~1; }
+
+// workspace layout (elements of cplx<T>); one right-hand side:
+//   t0 [m0 row] | B_l [n_l row] (l = 1..Lf) | t_l [m_l row] (l = 1..Lf-1) | P, Q of the odd levels,
+//   of the even levels | xf [row]
+// several: t0 [m0 row] | B_1 [n_1 row] | t_l [m_l row] (l = 1..Lf-1) | xf [row]
 static int64_t ws_elems(const BcrHandle* h, int nrhs) {
-  int64_t row = (int64_t)h->ny * nrhs;
-  int64_t tot = h->m[0] * row;
-  for (int l = 1; l <= h->Lf; ++l) tot += h->n[l] * row;
-  for (int l = 1; l < h->Lf; ++l) tot += h->m[l] * row;
-  int64_t m1 = h->Lf > 1 ? h->m[1] : 0, m2 = h->Lf > 2 ? h->m[2] : 0;
-  tot += 2 * m1 * row + 2 * m2 * row + row;  // P, Q of the odd levels, of the even levels, xf
-  return tot;
+  const int64_t row = (int64_t)h->ny * (nrhs == 1 ? 1 : ws_cols(h, nrhs));
+  int64_t t = 0, B = 0;
+  for (int l = 1; l <= h->Lf; ++l) B += h->n[l];
+  for (int l = 1; l < h->Lf; ++l) t += h->m[l];
+  if (nrhs > 1) return std::max((h->m[0] + h->n[1] + t + 1) * row, ws_elems(h, 1));
+  const int64_t m1 = h->Lf > 1 ? h->m[1] : 0, m2 = h->Lf > 2 ? h->m[2] : 0;
+  return (h->m[0] + B + t + 2 * m1 + 2 * m2 + 1) * row;
 }
 
 cudaError_t bcr_reserve_ws(BcrHandle* h, int nrhs) {
@@ -2466,9 +2458,283 @@ cudaError_t bcr_reserve_ws(BcrHandle* h, int nrhs) {
   return cudaSuccess;
 }
 
+// ===================================================================== several right-hand sides
+// The rows of every level live in one array B1 (level l: rows 2^(l-1) apart), so that a level's
+// kept rows are updated in place, the solution of a level is found where the level below reads
+// it, and no copies or separate sums remain:
+//   forward   t_k = Dinv_k b_{2k+1};  b_{2e} -= Y_{e-1}^T b_{2e-1} + X_e^T b_{2e+1}
+//   backward  x_{2k+1} = t_k - X_k x_{2k} - Y_k x_{2k+2}
+// Each line is one launch: FP32 on the TMA-fed tensor-core kernel (a product over two K segments),
+// FP64 on the digit split of tc_gemm64.cu; the SIMT pipe and sizes the split does not take run
+// the products one by one.
+namespace {
+
+// One level of the solve: dst_z = c0_z - A0_z[op] src_{z+z0} - A1_z[op] src_{z+z1} over the z that
+// have them; rows of src `ss`, of dst `sd`, of c0 `sc` elements apart.
 template <typename T>
-static cudaError_t solve_t(BcrHandle* h, const double2* cx, const cplx<T>* b, cplx<T>* x, int nrhs,
-                           cudaStream_t s) {
+struct MultiTerm {
+  const cplx<T>* A;   // null: the term is not there
+  int nA;             // members
+  bool ta;
+  int zA, zB, zlo, zhi;
+};
+
+}  // namespace
+
+template <typename T>
+static cudaError_t multi_update(BcrHandle* h, int ny, int nq, const MultiTerm<T> (&tm)[2], const cplx<T>* src,
+                                int64_t ss, int nsrc, const cplx<T>* c0, int64_t sc, cplx<T>* dst, int64_t sd,
+                                int batch, cudaStream_t s) {
+  const int64_t nn = (int64_t)ny * ny;
+  const cplx<T> one = mkc(T(1), T(0)), mone = mkc(T(-1), T(0));
+  if (batch <= 0) return cudaSuccess;
+  if constexpr (sizeof(T) == 4) {
+    if (!h->simt) {
+      TcJob j{};
+      for (const MultiTerm<T>& t : tm)
+        if (t.A && t.zhi > t.zlo)
+          j.seg[j.nseg++] = TcSegment{t.A, ny, nn, t.nA, t.ta, src, nq, ss, nsrc, false, ny, t.zA, t.zB, t.zlo, t.zhi};
+      if (j.nseg > 0) {
+        j.alpha = -1.f;
+        j.beta = 1.f;
+        j.C0 = c0;
+        j.ldc0 = nq;
+        j.sC0 = sc;
+        j.C = dst;
+        j.ldc = nq;
+        j.sC = sd;
+        j.batch = batch;
+        const cudaError_t e = launch_tc_cgemm_tma_jobs(ny, nq, 1, &j, h->status, tc_wait_limit(), s);
+        if (e != cudaErrorNotSupported) return e;
+      }
+    }
+  }
+  // one product after the other: the first takes c0 (it covers every row where c0 is not dst)
+  bool first = true;
+  for (const MultiTerm<T>& t : tm) {
+    if (!t.A || t.zhi <= t.zlo) continue;
+    const cplx<T>* c = first ? c0 + t.zlo * sc : dst + t.zlo * sd;
+    RCI_CUDA_TRY(gemm<T>(ny, nq, ny, t.ta, false, mone, t.A + (t.zlo + t.zA) * nn, ny, nn,
+                         src + (t.zlo + t.zB) * ss, nq, ss, one, c, nq, first ? sc : sd, dst + t.zlo * sd, nq, sd,
+                         t.zhi - t.zlo, s, nullptr, PF_SOLVE, gemm_status(h)));
+    first = false;
+  }
+  return cudaSuccess;
+}
+
+// blocks per batch of the FP64 split solve that the handle's scratch holds (0: not taken)
+static int split_solve_batch(const BcrHandle* h, int nq) {
+  const int ny = h->ny;
+  if (ny > SG_KMAX) return 0;
+  const size_t bytes = (size_t)std::max<int64_t>(h->m[0], 1) * ny * ny * sizeof(double2);
+  const size_t per = 3 * (sg_form_bytes(ny, ny, 3) + up256(4 * sg_form_exps(ny))) + sg_form_bytes(nq, ny, 2) +
+                     up256(4 * sg_form_exps(nq));
+  const size_t fixed = 2 * per + 16 * 256;  // one block more per form
+  return bytes <= fixed ? 0 : (int)std::min<size_t>((bytes - fixed) / per, 4096);
+}
+
+// One forward level in FP64: rows n of B (st elements apart), m eliminated.
+static cudaError_t split_fwd(BcrHandle* h, int cmax, const double2* Dinv, const double2* X, const double2* Y,
+                             double2* B, int64_t st, double2* t, int n, int m, int nk, int nq, cudaStream_t s) {
+  const int ny = h->ny, my = (n - 1) / 2;
+  const int64_t nn = (int64_t)ny * ny, row = (int64_t)ny * nq;
+  const size_t f3 = sg_form_bytes(ny, ny, 3), fb = sg_form_bytes(nq, ny, 2);
+  const int ne = sg_form_exps(ny), nb = sg_form_exps(nq);
+  const int cb = (int)ceil_div(nk, ceil_div(nk, cmax));
+  for (int k0 = 0; k0 < nk; k0 += cb) {
+    const int c = std::min(cb, nk - k0), cm = std::min(c, m - k0), p0 = k0 > 0 ? 1 : 0;
+    const int ny1 = std::max(0, std::min(k0 + c - 1, my) - (k0 - p0));  // Y of rows k0 - p0 .. k0 + c - 2
+    const int nb1 = p0 + cm;                                            // odd rows from index k0 - p0 on
+    Carve w{(unsigned char*)h->scratch};
+    unsigned char* fD = w.take<unsigned char>(c * f3);
+    unsigned char* fX = w.take<unsigned char>(c * f3);
+    unsigned char* fY = w.take<unsigned char>((c + 1) * f3);
+    unsigned char* fB = w.take<unsigned char>((c + 1) * fb);
+    int32_t* eD = w.take<int32_t>(4 * (size_t)ne * c);
+    int32_t* eX = w.take<int32_t>(4 * (size_t)ne * c);
+    int32_t* eY = w.take<int32_t>(4 * (size_t)ne * (c + 1));
+    int32_t* eB = w.take<int32_t>(4 * (size_t)nb * (c + 1));
+    RCI_CUDA_TRY(launch_sg_split(Dinv + k0 * nn, false, ny, nn, false, ny, ny, 3, cm, fD, eD, nullptr, s));
+    RCI_CUDA_TRY(launch_sg_split(X + k0 * nn, false, ny, nn, true, ny, ny, 3, cm, fX, eX, nullptr, s));
+    RCI_CUDA_TRY(launch_sg_split(Y + (k0 - p0) * nn, false, ny, nn, true, ny, ny, 3, ny1, fY, eY, nullptr, s));
+    RCI_CUDA_TRY(launch_sg_split(B + (2 * (int64_t)(k0 - p0) + 1) * st, false, nq, 2 * st, true, nq, ny, 2, nb1, fB,
+                                 eB, nullptr, s));
+    SgJob j[2] = {};
+    j[0].nseg = 1;
+    j[0].seg[0] = SgSeg{fD, eD, fB, eB, 3, 2, 0, p0, 0, cm};
+    j[0].C = t + k0 * row;
+    j[0].ldc = nq;
+    j[0].sC = row;
+    j[0].batch = cm;
+    j[1].nseg = 2;
+    j[1].seg[0] = SgSeg{fY, eY, fB, eB, 3, 2, p0 - 1, p0 - 1, 1 - p0, c};
+    j[1].seg[1] = SgSeg{fX, eX, fB, eB, 3, 2, 0, p0, 0, cm};
+    j[1].neg = true;
+    j[1].C = B + 2 * (int64_t)k0 * st;
+    j[1].ldc = nq;
+    j[1].sC = 2 * st;
+    j[1].C0 = j[1].C;
+    j[1].ldc0 = nq;
+    j[1].sC0 = 2 * st;
+    j[1].batch = c;
+    RCI_CUDA_TRY(launch_sg_gemm(ny, nq, ny, 2, j, SG_FULL, h->status, tc_wait_limit(), s));
+  }
+  return cudaSuccess;
+}
+
+// One backward level in FP64.
+static cudaError_t split_bwd(BcrHandle* h, int cmax, const double2* X, const double2* Y, double2* B, int64_t st,
+                             const double2* t, int n, int m, int nq, cudaStream_t s) {
+  const int ny = h->ny, my = (n - 1) / 2;
+  const int64_t nn = (int64_t)ny * ny, row = (int64_t)ny * nq;
+  const size_t f3 = sg_form_bytes(ny, ny, 3), fb = sg_form_bytes(nq, ny, 2);
+  const int ne = sg_form_exps(ny), nb = sg_form_exps(nq), nk = (n + 1) / 2;
+  const int cb = (int)ceil_div(m, ceil_div(m, cmax));
+  for (int k0 = 0; k0 < m; k0 += cb) {
+    const int c = std::min(cb, m - k0), cy = std::max(0, std::min(c, my - k0)), nb1 = std::min(c + 1, nk - k0);
+    Carve w{(unsigned char*)h->scratch};
+    unsigned char* fX = w.take<unsigned char>(c * f3);
+    unsigned char* fY = w.take<unsigned char>(c * f3);
+    unsigned char* fB = w.take<unsigned char>((c + 1) * fb);
+    int32_t* eX = w.take<int32_t>(4 * (size_t)ne * c);
+    int32_t* eY = w.take<int32_t>(4 * (size_t)ne * c);
+    int32_t* eB = w.take<int32_t>(4 * (size_t)nb * (c + 1));
+    RCI_CUDA_TRY(launch_sg_split(X + k0 * nn, false, ny, nn, false, ny, ny, 3, c, fX, eX, nullptr, s));
+    RCI_CUDA_TRY(launch_sg_split(Y + k0 * nn, false, ny, nn, false, ny, ny, 3, cy, fY, eY, nullptr, s));
+    RCI_CUDA_TRY(launch_sg_split(B + 2 * (int64_t)k0 * st, false, nq, 2 * st, true, nq, ny, 2, nb1, fB, eB, nullptr, s));
+    SgJob j{};
+    j.nseg = 2;
+    j.seg[0] = SgSeg{fX, eX, fB, eB, 3, 2, 0, 0, 0, c};
+    j.seg[1] = SgSeg{fY, eY, fB, eB, 3, 2, 0, 1, 0, cy};
+    j.neg = true;
+    j.C0 = t + k0 * row;
+    j.ldc0 = nq;
+    j.sC0 = row;
+    j.C = B + (2 * (int64_t)k0 + 1) * st;
+    j.ldc = nq;
+    j.sC = 2 * st;
+    j.batch = c;
+    RCI_CUDA_TRY(launch_sg_gemm(ny, nq, ny, 1, &j, SG_FULL, h->status, tc_wait_limit(), s));
+  }
+  return cudaSuccess;
+}
+
+template <typename T>
+static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b, cplx<T>* x, int nrhs,
+                               cudaStream_t s) {
+  const int nx = h->nx, ny = h->ny, nq = ws_cols(h, nrhs);
+  const int64_t nn = (int64_t)ny * ny, row = (int64_t)ny * nq;
+  const int m0 = (int)h->m[0], n1 = (nx + 1) / 2;
+  RCI_CUDA_TRY(bcr_reserve_ws(h, nrhs));
+  cplx<T>* p = (cplx<T>*)h->ws;
+  cplx<T>* t0 = p;
+  p += m0 * row;
+  cplx<T>* B1 = p;
+  p += n1 * row;
+  std::vector<cplx<T>*> tl(h->Lf + 1, nullptr);
+  for (int l = 1; l < h->Lf; ++l) {
+    tl[l] = p;
+    p += h->m[l] * row;
+  }
+  cplx<T>* xf = p;
+  auto store = (const cplx<T>*)h->store;
+  const cplx<T> one = mkc(T(1), T(0)), zero = czero<T>();
+  double sbytes = 2.0 * m0 * 5.0 * ny * sizeof(cplx<T>), sflops = 2.0 * 30.0 * m0 * (double)ny * nrhs;
+  for (int l = 1; l < h->Lf; ++l) {
+    sbytes += 5.0 * h->m[l] * (double)nn * sizeof(cplx<T>);
+    sflops += 5.0 * 8.0 * h->m[l] * (double)nn * nrhs;
+  }
+  sbytes += (double)nn * sizeof(cplx<T>) + 2.0 * nx * (double)ny * nrhs * sizeof(cplx<T>);
+  const int dense = h->Lf - 1;
+  ProfScope ps(h->prof, PF_SOLVE, s, sflops, sbytes, (m0 > 0 ? 1 : 0) + 1 + 2 * dense + 1 + dense + 1);
+  int cmax = 0;
+  if constexpr (sizeof(T) == 8) cmax = split_solve_batch(h, nq);
+
+  // ---- level 0 forward by tridiagonal sweeps, then its kept rows
+  if (m0 > 0) {
+    fwd0_kernel<T><<<(unsigned)ceil_div((int64_t)m0 * nrhs, 128), 128, 0, s>>>(
+        b, t0, ny, m0, nrhs, nq, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+        (const cplx<T>*)h->tdu2, h->tpiv);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+  }
+  keep0_kernel<T><<<(unsigned)ceil_div(n1 * row, 256), 256, 0, s>>>(b, t0, cx, B1, nx, ny, n1, nrhs, nq);
+  rci_note_launch();
+  RCI_CUDA_TRY(cudaGetLastError());
+  // ---- dense levels forward
+  for (int l = 1; l < h->Lf; ++l) {
+    const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1], my = (n - 1) / 2;
+    const cplx<T>* Dinv = store + h->off[l];
+    const cplx<T>* X = Dinv + (int64_t)m * nn;
+    const cplx<T>* Y = X + (int64_t)m * nn;
+    const int64_t st = row << (l - 1);
+    if constexpr (sizeof(T) == 8) {
+      if (cmax > 0) {
+        RCI_CUDA_TRY(split_fwd(h, cmax, Dinv, X, Y, B1, st, tl[l], n, m, nk, nq, s));
+        continue;
+      }
+    }
+    RCI_CUDA_TRY(gemm<T>(ny, nq, ny, false, false, one, Dinv, ny, nn, B1 + st, nq, 2 * st, zero, nullptr, 0, 0,
+                         tl[l], nq, row, m, s, nullptr, PF_SOLVE, gemm_status(h)));
+    const MultiTerm<T> tm[2] = {{Y, my, true, -1, -1, 1, my + 1}, {X, m, true, 0, 0, 0, m}};
+    RCI_CUDA_TRY(multi_update<T>(h, ny, nq, tm, B1 + st, 2 * st, m, B1, 2 * st, B1, 2 * st, nk, s));
+  }
+  // ---- single remaining row
+  {
+    const cplx<T>* Dinv = store + h->final_off;
+    bool done = false;
+    if constexpr (sizeof(T) == 8) {
+      if (cmax > 0) {
+        Carve w{(unsigned char*)h->scratch};
+        unsigned char* fD = w.take<unsigned char>(sg_form_bytes(ny, ny, 3));
+        unsigned char* fB = w.take<unsigned char>(sg_form_bytes(nq, ny, 2));
+        int32_t* eD = w.take<int32_t>(4 * (size_t)sg_form_exps(ny));
+        int32_t* eB = w.take<int32_t>(4 * (size_t)sg_form_exps(nq));
+        RCI_CUDA_TRY(launch_sg_split(Dinv, false, ny, nn, false, ny, ny, 3, 1, fD, eD, nullptr, s));
+        RCI_CUDA_TRY(launch_sg_split(B1, false, nq, row, true, nq, ny, 2, 1, fB, eB, nullptr, s));
+        SgJob j{};
+        j.nseg = 1;
+        j.seg[0] = SgSeg{fD, eD, fB, eB, 3, 2, 0, 0, 0, 1};
+        j.C = B1;  // (the operand is its split form)
+        j.ldc = nq;
+        j.sC = row;
+        j.batch = 1;
+        RCI_CUDA_TRY(launch_sg_gemm(ny, nq, ny, 1, &j, SG_FULL, h->status, tc_wait_limit(), s));
+        done = true;
+      }
+    }
+    if (!done) {
+      RCI_CUDA_TRY(gemm<T>(ny, nq, ny, false, false, one, Dinv, ny, 0, B1, nq, 0, zero, nullptr, 0, 0, xf, nq, 0, 1, s,
+                           nullptr, PF_SOLVE, gemm_status(h)));
+      RCI_CUDA_TRY(cudaMemcpyAsync(B1, xf, row * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
+    }
+  }
+  // ---- dense levels backward
+  for (int l = h->Lf - 1; l >= 1; --l) {
+    const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1], my = (n - 1) / 2;
+    const cplx<T>* X = store + h->off[l] + (int64_t)m * nn;
+    const cplx<T>* Y = X + (int64_t)m * nn;
+    const int64_t st = row << (l - 1);
+    if constexpr (sizeof(T) == 8) {
+      if (cmax > 0) {
+        RCI_CUDA_TRY(split_bwd(h, cmax, X, Y, B1, st, tl[l], n, m, nq, s));
+        continue;
+      }
+    }
+    const MultiTerm<T> tm[2] = {{X, m, false, 0, 0, 0, m}, {Y, my, false, 0, 1, 0, my}};
+    RCI_CUDA_TRY(multi_update<T>(h, ny, nq, tm, B1, 2 * st, nk, tl[l], row, B1 + st, 2 * st, m, s));
+  }
+  // ---- level 0 backward by tridiagonal sweeps (and the kept rows copied)
+  bwd0_kernel<T><<<(unsigned)ceil_div((int64_t)n1 * nrhs, 128), 128, 0, s>>>(
+      b, B1, cx, x, nx, ny, n1, nrhs, nq, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+      (const cplx<T>*)h->tdu2, h->tpiv);
+  rci_note_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, cplx<T>* x, cudaStream_t s) {
+  constexpr int nrhs = 1;
   const int nx = h->nx, ny = h->ny;
   const int64_t nn = (int64_t)ny * ny;
   const int64_t row = (int64_t)ny * nrhs;
@@ -2501,28 +2767,18 @@ static cudaError_t solve_t(BcrHandle* h, const double2* cx, const cplx<T>* b, cp
   cplx<T>* xf = p;
 
   auto store = (const cplx<T>*)h->store;
-  const cplx<T>* G0 = (const cplx<T>*)h->G0;
-  const cplx<T> one = mkc(T(1), T(0)), mone = mkc(T(-1), T(0)), zero = czero<T>();
 
-  // level 0: the tridiagonal factors twice for one right-hand side (dense inverses G0 for
-  // several); levels >= 1: Dinv, X, Y forward and X, Y backward
-  double sbytes = nrhs == 1 ? 2.0 * m0 * 5.0 * ny * sizeof(cplx<T>) : 2.0 * m0 * (double)nn * sizeof(cplx<T>);
-  double sflops = nrhs == 1 ? 2.0 * 30.0 * m0 * (double)ny : 2.0 * 8.0 * m0 * (double)nn * nrhs;
+  // level 0: the tridiagonal factors twice; levels >= 1: Dinv, X, Y forward and X, Y backward
+  double sbytes = 2.0 * m0 * 5.0 * ny * sizeof(cplx<T>), sflops = 2.0 * 30.0 * m0 * (double)ny;
   for (int l = 1; l < h->Lf; ++l) {
     sbytes += 5.0 * h->m[l] * (double)nn * sizeof(cplx<T>);
-    sflops += 5.0 * 8.0 * h->m[l] * (double)nn * nrhs;
+    sflops += 5.0 * 8.0 * h->m[l] * (double)nn;
   }
-  sbytes += (double)nn * sizeof(cplx<T>) + 2.0 * nx * (double)ny * nrhs * sizeof(cplx<T>);
-  ProfScope ps(h->prof, PF_SOLVE, s, sflops, sbytes, 0);
-  // kernels this solve launches (level-0 pair, per dense level forward and backward, the
-  // single remaining row); several right-hand sides run the level products as GEMMs
-  {
-    const int dense = h->Lf - 1, l0 = m0 > 0 ? 1 : 0;
-    ps.nl = nrhs == 1 ? l0 + 1 + dense + 1 + dense + 1
-                      : l0 + 1 + 4 * dense + 1 + 3 * dense + 1 + l0;
-  }
+  sbytes += (double)nn * sizeof(cplx<T>) + 2.0 * nx * (double)ny * sizeof(cplx<T>);
+  // kernels launched: level-0 pair, per dense level forward and backward, the last row
+  const int dense = h->Lf - 1, l0 = m0 > 0 ? 1 : 0;
+  ProfScope ps(h->prof, PF_SOLVE, s, sflops, sbytes, l0 + 1 + dense + 1 + dense + 1);
 
-  if (nrhs == 1) {
     if (ny % vec16<T>::per != 0 || ny > 256 * vec16<T>::per)
       return cudaErrorInvalidValue;  // (grid creation keeps ny within these limits)
     const int smax = (int)ceil_div(ny, 32 * vec16<T>::per);
@@ -2565,7 +2821,7 @@ static cudaError_t solve_t(BcrHandle* h, const double2* cx, const cplx<T>* b, cp
     }
     {
       int64_t nt = (int64_t)n1 * row;
-      keep0_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(bsrc, t0, cx, B[1], nx, ny, n1, 1);
+      keep0_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(bsrc, t0, cx, B[1], nx, ny, n1, 1, 1);
       rci_note_launch();
       RCI_CUDA_TRY(cudaGetLastError());
     }
@@ -2617,87 +2873,6 @@ static cudaError_t solve_t(BcrHandle* h, const double2* cx, const cplx<T>* b, cp
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
 #undef RCI_SMAX_DISPATCH
-    return cudaSuccess;
-  }
-
-  // ================= several right-hand sides: batched GEMMs per level
-  // ---- the stored inverses of level 0, formed once per factorisation
-  if (m0 > 0 && !h->g0_valid) {
-    const int thr = (int)ceil_div(ny, 32) * 32;
-    const size_t smem = l0_smem<T>(ny);
-    if (smem > 48 * 1024)
-      RCI_CUDA_TRY(cudaFuncSetAttribute(level0_schur_kernel<T, 1>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    cplx<T>* g0w = (cplx<T>*)h->G0;
-    level0_schur_kernel<T, 1><<<m0, thr, smem, s>>>(nullptr, nullptr, nullptr, nx, ny,
-                                                    (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv,
-                                                    (const cplx<T>*)h->tdu, (const cplx<T>*)h->tdu2,
-                                                    h->tpiv, g0w, g0w, g0w, g0w, g0w);
-    rci_note_launch();
-    RCI_CUDA_TRY(cudaGetLastError());
-    h->g0_valid = true;
-  }
-  // ---- level 0 forward: t0[k] = T_{2k+1}^{-1} b[2k+1] with the stored inverses
-  if (m0 > 0)
-    RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, false, false, one, G0, ny, nn, b + row, nrhs, 2 * row, zero,
-                         nullptr, 0, 0, t0, nrhs, row, m0, s, nullptr, PF_SOLVE, gemm_status(h)));
-  {
-    int64_t nt = (int64_t)n1 * row;
-    keep0_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(b, t0, cx, B[1], nx, ny, n1, nrhs);
-    rci_note_launch();
-    RCI_CUDA_TRY(cudaGetLastError());
-  }
-  // ---- dense levels forward
-  for (int l = 1; l < h->Lf; ++l) {
-    const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
-    const int my = (n - 1) / 2;
-    const cplx<T>* Dinv = store + h->off[l];
-    const cplx<T>* X = Dinv + (int64_t)m * nn;
-    const cplx<T>* Y = X + (int64_t)m * nn;
-    const cplx<T>* Bodd = B[l] + row;
-    RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, false, false, one, Dinv, ny, nn, Bodd, nrhs, 2 * row, zero,
-                         nullptr, 0, 0, tl[l], nrhs, row, m, s, nullptr, PF_SOLVE, gemm_status(h)));
-    RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, true, false, one, X, ny, nn, Bodd, nrhs, 2 * row, zero,
-                         nullptr, 0, 0, P, nrhs, row, m, s, nullptr, PF_SOLVE, gemm_status(h)));
-    RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, true, false, one, Y, ny, nn, Bodd, nrhs, 2 * row, zero,
-                         nullptr, 0, 0, Q, nrhs, row, my, s, nullptr, PF_SOLVE, gemm_status(h)));
-    int64_t nt = (int64_t)nk * row;
-    keep_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(B[l], P, Q, B[l + 1], m, nk, row);
-    rci_note_launch();
-    RCI_CUDA_TRY(cudaGetLastError());
-  }
-  // ---- single remaining row
-  RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, false, false, one, store + h->final_off, ny, 0, B[h->Lf], nrhs,
-                       0, zero, nullptr, 0, 0, xf, nrhs, 0, 1, s, nullptr, PF_SOLVE, gemm_status(h)));
-  RCI_CUDA_TRY(cudaMemcpyAsync(B[h->Lf], xf, row * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
-  // ---- dense levels backward (the solution of level l overwrites B[l])
-  for (int l = h->Lf - 1; l >= 1; --l) {
-    const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
-    const int my = (n - 1) / 2;
-    const cplx<T>* Dinv = store + h->off[l];
-    const cplx<T>* X = Dinv + (int64_t)m * nn;
-    const cplx<T>* Y = X + (int64_t)m * nn;
-    int64_t nt = (int64_t)nk * row;
-    copy_kept_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(B[l + 1], B[l], nk, row);
-    rci_note_launch();
-    RCI_CUDA_TRY(cudaGetLastError());
-    RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, false, false, mone, X, ny, nn, B[l + 1], nrhs, row, one,
-                         tl[l], nrhs, row, B[l] + row, nrhs, 2 * row, m, s, nullptr, PF_SOLVE, gemm_status(h)));
-    RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, false, false, mone, Y, ny, nn, B[l + 1] + row, nrhs, row,
-                         one, B[l] + row, nrhs, 2 * row, B[l] + row, nrhs, 2 * row, my, s, nullptr, PF_SOLVE, gemm_status(h)));
-  }
-  // ---- level 0 backward: x[2k+1] = T^{-1}(b[2k+1] - couplings x), stored inverses
-  {
-    int64_t nt = (int64_t)n1 * row;
-    // t0 (no longer needed) holds the eliminated rows' right-hand sides
-    bwd0_rhs_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(b, B[1], cx, x, t0, nx, ny, n1,
-                                                                    nrhs);
-    rci_note_launch();
-    RCI_CUDA_TRY(cudaGetLastError());
-    if (m0 > 0)
-      RCI_CUDA_TRY(gemm<T>(ny, nrhs, ny, false, false, one, G0, ny, nn, t0, nrhs, row, zero,
-                           nullptr, 0, 0, x + row, nrhs, 2 * row, m0, s, nullptr, PF_SOLVE, gemm_status(h)));
-  }
   return cudaSuccess;
 }
 
@@ -2705,8 +2880,10 @@ cudaError_t bcr_solve(BcrHandle* h, const double2* cx, const void* b, void* x, i
                       cudaStream_t s) {
   if (nrhs < 1) return cudaErrorInvalidValue;
   if (h->prec == RCI_FP64)
-    return solve_t<double>(h, cx, (const double2*)b, (double2*)x, nrhs, s);
-  return solve_t<float>(h, cx, (const float2*)b, (float2*)x, nrhs, s);
+    return nrhs == 1 ? solve_one<double>(h, cx, (const double2*)b, (double2*)x, s)
+                     : solve_multi<double>(h, cx, (const double2*)b, (double2*)x, nrhs, s);
+  return nrhs == 1 ? solve_one<float>(h, cx, (const float2*)b, (float2*)x, s)
+                   : solve_multi<float>(h, cx, (const float2*)b, (float2*)x, nrhs, s);
 }
 
 cudaError_t bcr_block_inverse(const void* src, void* out, int n, int batch, int prec, int kernel,
@@ -2739,6 +2916,7 @@ cudaError_t bcr_gemm(int M, int N, int K, bool ta, bool tb, double alpha, const 
       return launch_tc_cgemm(M, N, K, ta, tb, al, a, lda, sA, b, ldb, sB, be, c0, ldc0, sC0, c, ldc,
                              sC, batch, status, s, 1);
     case 2: {
+      if (N > 160) return cudaErrorInvalidValue;  // (the entry point's stated limit)
       const cudaError_t e = launch_tc_cgemm_tma(M, N, K, ta, tb, (float)alpha, a, lda, sA, b, ldb, sB,
                                                 (float)beta, c0, ldc0, sC0, c, ldc, sC, batch,
                                                 status, tc_wait_limit(), s);

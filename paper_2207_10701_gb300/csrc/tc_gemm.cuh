@@ -6,7 +6,7 @@
 // C[z] = alpha op(A[z]) op(B[z]) + beta C0[z] for z < batch (row-major complex64,
 // element strides between batch members).  Bounded internal waits: a timeout is
 // recorded as DEV_TIMEOUT in *status.
-// variant: 0 = the TMA-fed kernel where it applies (real alpha, beta, N <= 160, the
+// variant: 0 = the TMA-fed kernel where it applies (real alpha, beta, N even, the
 // alignments below), else the register-staged kernels; 1 = register-staged only.
 cudaError_t launch_tc_cgemm(int M, int N, int K, bool ta, bool tb, float2 alpha, const float2* A,
                             int64_t lda, int64_t sA, const float2* B, int64_t ldb, int64_t sB,
@@ -14,7 +14,7 @@ cudaError_t launch_tc_cgemm(int M, int N, int K, bool ta, bool tb, float2 alpha,
                             int64_t ldc, int64_t sC, int batch, int32_t* status, cudaStream_t s,
                             int variant = 0);
 
-// The TMA-fed form (tc_gemm_tma.cu): real alpha and beta, 2 <= N <= 160 and even, A, B, C,
+// The TMA-fed form (tc_gemm_tma.cu): real alpha and beta, N even, A, B, C,
 // C0 16-byte aligned, even leading dimensions and batch strides.  Returns
 // cudaErrorNotSupported (nothing launched) where these do not hold.
 cudaError_t launch_tc_cgemm_tma(int M, int N, int K, bool ta, bool tb, float alpha,

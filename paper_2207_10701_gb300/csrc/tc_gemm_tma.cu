@@ -1,7 +1,7 @@
 // Batched complex FP32 GEMM on the 5th-generation tensor cores, fed by the Tensor Memory
 // Accelerator, with the A operand in tensor memory (3xTF32, real alpha and beta):
 //
-//   C[z] = alpha op(A[z]) op(B[z]) + beta C0[z]      (row-major complex64, N <= 160)
+//   C[z] = alpha op(A[z]) op(B[z]) + beta C0[z]      (row-major complex64)
 //
 // Algebra (as the shared-memory kernels in tc_gemm.cu): the complex product is the real
 // product of the stacked A_s (rows (ar, -ai) and (ai, ar) per complex k) with B_s (rows
@@ -53,7 +53,7 @@ namespace {
 
 constexpr int TT_ROWS = 64;       // complex rows per tile (128 tensor-memory lanes)
 constexpr int TT_KC = 8;          // complex k per stage
-constexpr int TT_NMAX = 160;      // largest N (complex columns)
+constexpr int TT_NMAX = 160;      // most columns of a tile
 #ifndef RCI_TMA_RAW_STAGES
 #define RCI_TMA_RAW_STAGES 4
 #endif
@@ -123,7 +123,8 @@ struct TtJob {
 };
 
 struct TtArgs {
-  int M, N, NB;     // NB: N rounded up to 16 (the MMA's N)
+  int M, N;
+  int NB, ntn;      // columns per tile (a multiple of 16, the MMA's N), column tiles
   int njob, ntiles;
   TtJob job[2];
   int32_t* status;
@@ -150,18 +151,20 @@ __device__ __forceinline__ const CUtensorMap* map_at(const TtMaps& maps, int i) 
 }
 
 struct TtTile {
-  int j, z, i0;     // job, product within the job, first row
+  int j, z, i0, n0;  // job, product within the job, first row, first column
 };
 
 // (jobs: the launch's jobs copied to shared memory: reading the job of a tile straight from
 // the kernel parameter at a run-time index gave wrong rows in the library build, and the
 // tensor maps are taken at constant offsets for the same reason)
-__device__ __forceinline__ TtTile tile_of(const TtJob* jobs, int njob, int tile, int mt) {
+__device__ __forceinline__ TtTile tile_of(const TtJob* jobs, const TtArgs& p, int tile, int mt) {
   TtTile t;
-  t.j = (njob > 1 && tile >= jobs[1].tile0) ? 1 : 0;
+  t.j = (p.njob > 1 && tile >= jobs[1].tile0) ? 1 : 0;
   const int local = tile - jobs[t.j].tile0;
-  t.z = local / mt;
-  t.i0 = (local - t.z * mt) * TT_ROWS;
+  const int zm = local / p.ntn;
+  t.n0 = (local - zm * p.ntn) * p.NB;
+  t.z = zm / mt;
+  t.i0 = (zm - t.z * mt) * TT_ROWS;
   return t;
 }
 
@@ -291,6 +294,13 @@ __device__ __forceinline__ void mma_tf32_ta(uint32_t d, uint32_t a_tmem, uint64_
       "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
+// one lane of a converged warp, known to the compiler as one
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0u;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -394,7 +404,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
       int it = 0;
       bool ok = true;
       for (int tl = 0; tl < ntl && ok; ++tl) {
-        const TtTile t = tile_of(jobs, p.njob, (int)blockIdx.x + tl * (int)gridDim.x, mt);
+        const TtTile t = tile_of(jobs, p, (int)blockIdx.x + tl * (int)gridDim.x, mt);
         const TtJob& q = jobs[t.j];
         bool v0, v1;
         const int nst = tile_stages(q, t.z, v0, v1);
@@ -417,8 +427,8 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
           mbar_expect_tx(&raw_full[s], bytes);
           if (!sg.ta) tma_load_3d(ra, mA, k0, t.i0, za, &raw_full[s]);
           else tma_load_3d(ra, mA, t.i0, k0, za, &raw_full[s]);
-          if (!sg.tb) tma_load_3d(rb, mB, 0, k0, zb, &raw_full[s]);
-          else tma_load_3d(rb, mB, k0, 0, zb, &raw_full[s]);
+          if (!sg.tb) tma_load_3d(rb, mB, t.n0, k0, zb, &raw_full[s]);
+          else tma_load_3d(rb, mB, k0, t.n0, zb, &raw_full[s]);
         }
       }
       // the copies lane 0 issued land before the CTA can exit
@@ -452,7 +462,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     int it = 0;
     bool ok = true;
     for (int tl = 0; tl < ntl && ok; ++tl) {
-      const TtTile t = tile_of(jobs, p.njob, (int)blockIdx.x + tl * (int)gridDim.x, mt);
+      const TtTile t = tile_of(jobs, p, (int)blockIdx.x + tl * (int)gridDim.x, mt);
       const TtJob& q = jobs[t.j];
       bool v0, v1;
       const int nst = tile_stages(q, t.z, v0, v1);
@@ -540,7 +550,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     }
   } else if (warp == TT_MMA_WARP) {
     // ------------------------------------------------------------ MMA issue
-    // (the warp waits together; lane 0 issues the MMAs and commits)
+    // (the warp waits together; one elected lane, always the same, issues the MMAs and commits)
     const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(NB >> 3) << 17) |
                            ((uint32_t)(128 >> 4) << 24);
     bool ok = true;
@@ -552,7 +562,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
         break;
       fence_after();
       const uint32_t acc = tmem + (uint32_t)b * TT_ACC_STRIDE;
-      const TtTile t = tile_of(jobs, p.njob, (int)blockIdx.x + tl * (int)gridDim.x, mt);
+      const TtTile t = tile_of(jobs, p, (int)blockIdx.x + tl * (int)gridDim.x, mt);
       bool v0, v1;
       const int nst = tile_stages(jobs[t.j], t.z, v0, v1);
       for (int st = 0; st < nst; ++st, ++it) {
@@ -562,7 +572,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
           break;
         }
         fence_after();
-        if (lane == 0) {
+        if (elect_one()) {
           const uint32_t aslot = tmem + a_slot(cs);
           const uint32_t bh = smem_u32(sm_raw + TT_CONV_OFF + (size_t)cs * TT_CSTAGE);
           const uint32_t bl = bh + TT_BSPLIT;
@@ -578,11 +588,11 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
         }
         __syncwarp();
       }
-      if (ok && lane == 0) mma_commit(&acc_full[b]);
+      if (ok && elect_one()) mma_commit(&acc_full[b]);
       __syncwarp();
     }
-    // every MMA issued by lane 0 has finished before the tensor memory is freed
-    if (lane == 0) {
+    // every MMA issued by the elected lane has finished before the tensor memory is freed
+    if (elect_one()) {
       mma_commit(done_bar);
       if (!tt_wait_own(done_bar, 0)) *abort_flag = 1;
     }
@@ -596,7 +606,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
     const int nch = NB / 16;
     for (int tl = 0; tl < ntl; ++tl) {
       const int b = tl & 1;
-      const TtTile t = tile_of(jobs, p.njob, (int)blockIdx.x + tl * (int)gridDim.x, mt);
+      const TtTile t = tile_of(jobs, p, (int)blockIdx.x + tl * (int)gridDim.x, mt);
       const TtJob& qj = jobs[t.j];
       const bool has_c0 = qj.C0 != nullptr && qj.beta != 0.f;
       const float alpha = qj.alpha, beta = qj.beta;
@@ -610,7 +620,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
       auto load_c0 = [&](int c, float4 (&dst)[4]) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int col = 16 * c + 4 * j + 2 * part;
+          const int col = t.n0 + 16 * c + 4 * j + 2 * part;
           dst[j] = (has_c0 && rok && col < p.N)
                        ? *reinterpret_cast<const float4*>(C0row + col)
                        : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -646,7 +656,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1)
           const float r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
           float4 o = part ? make_float4(r0, v[4 * j + 2], r1, v[4 * j + 3])
                           : make_float4(v[4 * j], r0, v[4 * j + 1], r1);
-          const int col = 16 * c + 4 * j + 2 * part;
+          const int col = t.n0 + 16 * c + 4 * j + 2 * part;
           if (rok && col < p.N) {
             o.x *= alpha;
             o.y *= alpha;
@@ -759,15 +769,17 @@ bool seg_maps(const TcSegment& g, int M, int N, int NB, CUtensorMap* mA, CUtenso
 cudaError_t launch_tc_cgemm_tma_jobs(int M, int N, int njob, const TcJob* jobs, int32_t* status,
                                      long long wait_limit, cudaStream_t s) {
   // the shapes and alignments the TMA boxes and the 16-byte epilogue stores need
-  if (M < 1 || N < 2 || N > TT_NMAX || (N & 1) || njob < 1 || njob > 2)
-    return cudaErrorNotSupported;
-  const int NB = (N + 15) & ~15;
+  if (M < 1 || N < 2 || (N & 1) || njob < 1 || njob > 2) return cudaErrorNotSupported;
+  // equal column tiles of at most TT_NMAX
+  const int NB = (int)ceil_div(ceil_div(N, ceil_div(N, TT_NMAX)), 16) * 16;
+  const int ntn = (int)ceil_div(N, NB);
   const int mt = (M + TT_ROWS - 1) / TT_ROWS;
   TtMaps maps{};
   TtArgs a{};
   a.M = M;
   a.N = N;
   a.NB = NB;
+  a.ntn = ntn;
   a.status = status;
   a.wait_limit = wait_limit;
   int64_t ntiles = 0;
@@ -801,10 +813,11 @@ cudaError_t launch_tc_cgemm_tma_jobs(int M, int N, int njob, const TcJob* jobs, 
     q.sC0 = jo.sC0;
     q.alpha = jo.alpha;
     q.beta = jo.beta;
-    ntiles += (int64_t)jo.batch * mt;
+    ntiles += (int64_t)jo.batch * mt * ntn;
     ++a.njob;
   }
   if (a.njob == 0) return cudaSuccess;
+  if (ntiles > 0x7fffffffLL) return cudaErrorNotSupported;
   a.ntiles = (int)ntiles;
   const unsigned grid = (unsigned)(ntiles < sms() ? ntiles : sms());
   RCI_CUDA_TRY(cudaFuncSetAttribute(tc_cgemm_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
