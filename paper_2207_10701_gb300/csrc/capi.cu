@@ -358,14 +358,16 @@ rci_status ensure_multi(rci_grid* g, int nq) {
   return RCI_OK;
 }
 
-// Residual r = b - A x (FP64 stencil) and the largest ||r||/||b|| over the columns.
+// Residual r = b - A x (FP64 stencil) and the largest ||r||/||b|| over the columns.  same_b: b is
+// that of the call before, whose ||b|| stands (several right-hand sides).
 rci_status residual_ratio(rci_grid* g, const double2* b, const double2* x, double2* r, int nrhs,
-                          double* worst) {
+                          double* worst, bool same_b = false) {
   int nblk = residual_blocks(g->g);
   {
     ProfScope ps(&g->prof, PF_RESIDUAL, g->s, 18.0 * g->N * nrhs,
                  (double)g->N * (48.0 + 48.0 * nrhs), 2);
-    CK(launch_residual(g->g, g->dg, g->cx, g->cy, b, x, r, nrhs, g->part_r, g->part_b, g->s),
+    CK(launch_residual(g->g, g->dg, g->cx, g->cy, b, x, r, nrhs, g->part_r,
+                       nrhs > 1 && same_b ? nullptr : g->part_b, g->s),
        "residual");
     CK(launch_ratio_norms(g->part_r, g->part_b, nblk, nrhs, g->ratio, g->s), "residual norms");
   }
@@ -397,7 +399,7 @@ rci_status solve64(rci_grid* g, BcrHandle* h, const double2* b, double2* x, doub
     CK(bcr_solve(h, g->cx, r, d, nrhs, g->s), "refine solve");
     CK(launch_axpy64(x, d, n, g->s), "refine update");
     ++*it;
-    st = residual_ratio(g, b, x, r, nrhs, worst);
+    st = residual_ratio(g, b, x, r, nrhs, worst, true);
     if (st != RCI_OK) return st;
   }
   return RCI_OK;
@@ -613,15 +615,15 @@ rci_status fp32_refine(rci_grid* g, const double2* b, double2* x, double2* r, vo
   const int64_t n = g->N * nrhs;
   int it = 0, kry = 0;
   *need64 = false;
-  CK(cudaMemsetAsync(x, 0, sizeof(double2) * n, g->s), "zero x");
-  CK(cudaMemcpyAsync(r, b, sizeof(double2) * n, cudaMemcpyDeviceToDevice, g->s), "copy b");
   double prev = 1.0;
   while (true) {
-    CK(launch_to_f32(r, (float2*)a32, n, g->s), "to fp32");
+    // the first solve starts from x = 0, whose residual is b
+    CK(launch_to_f32(it == 0 ? b : r, (float2*)a32, n, g->s), "to fp32");
     CK(bcr_solve(g->bcr, g->cx, a32, b32, nrhs, g->s), "fp32 solve");
-    CK(launch_add_f32(x, (const float2*)b32, n, g->s), "update");
+    if (it == 0) CK(launch_to_f64((const float2*)b32, x, n, g->s), "update");
+    else CK(launch_add_f32(x, (const float2*)b32, n, g->s), "update");
     ++it;
-    rci_status st = residual_ratio(g, b, x, r, nrhs, worst);
+    rci_status st = residual_ratio(g, b, x, r, nrhs, worst, it > 1);
     if (st == RCI_ENUMERIC) {
       *need64 = true;
       break;

@@ -22,7 +22,8 @@ cudaError_t launch_pml_coefficients(const GridGeom& g, double2* dg0, double2* ks
 cudaError_t launch_apply_A(const GridGeom& g, const double2* dg, const double2* cx,
                            const double2* cy, const double2* x, double2* y, int nrhs,
                            cudaStream_t s);
-// r = b - A x and per-RHS partial sums of |r|^2 and |b|^2 (nblk x nrhs each)
+// r = b - A x and per-RHS partial sums of |r|^2 and |b|^2 (nblk x nrhs each; several right-hand
+// sides: part_b null leaves the sums of an earlier call on the same b)
 int residual_blocks(const GridGeom& g);
 cudaError_t launch_residual(const GridGeom& g, const double2* dg, const double2* cx,
                             const double2* cy, const double2* b, const double2* x, double2* r,
