@@ -1429,22 +1429,14 @@ rci_status rci_qform_toeplitz(const double* v, const double* lags, int64_t n, do
                               void* stream) {
   if (!v || !lags || !out || n < 1 || n > (1LL << 31)) return RCI_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;
-  double* part = nullptr;
-  double* dout = nullptr;
-  size_t np = (size_t)qform_num_partials(n);
-  if (cudaMalloc(&part, sizeof(double) * np) != cudaSuccess) return RCI_ENOMEM;
-  if (cudaMalloc(&dout, sizeof(double)) != cudaSuccess) {
-    cudaFree(part);
-    return RCI_ENOMEM;
-  }
-  rci_status st = RCI_OK;
-  double F = 0.0;
-  if (launch_qform((const double2*)v, lags, n, part, dout, s) != cudaSuccess ||
-      cudaMemcpyAsync(&F, dout, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    st = RCI_ECUDA;
-  cudaFree(part);
-  cudaFree(dout);
+  QformWs w;
+  const cudaError_t e = qform_borrow(&w, n);
+  if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? RCI_ENOMEM : RCI_ECUDA;
+  const bool launched = launch_qform((const double2*)v, lags, n, w.part, w.result, s) == cudaSuccess;
+  const bool done = cudaStreamSynchronize(s) == cudaSuccess;
+  const rci_status st = launched && done ? RCI_OK : RCI_ECUDA;
+  const double F = st == RCI_OK ? *w.result : 0.0;
+  qform_return(w, done);
   if (st == RCI_OK) {
     if (!std::isfinite(F)) return RCI_ENUMERIC;
     *out = F;

@@ -120,3 +120,13 @@ cudaError_t launch_gather_source_col(const GridGeom& g, const double2* X, int ld
 int64_t qform_num_partials(int64_t n);
 cudaError_t launch_qform(const double2* v, const double* lags, int64_t n, double* partials,
                          double* out_dev, cudaStream_t s);
+// workspace of one rci_qform_toeplitz call (partials on the device, the result in pinned host
+// memory), lent until it is returned; ok: the stream that used it has been synchronised
+struct QformWs {
+  double* part = nullptr;
+  double* result = nullptr;
+  int device = 0;
+  bool kept = false;  // of the size that is kept between calls
+};
+cudaError_t qform_borrow(QformWs* w, int64_t n);
+void qform_return(const QformWs& w, bool ok);

@@ -5,13 +5,19 @@
 // and the Toeplitz matrix symmetric).  Per pair two FP64 FMAs: the block accumulates
 // s_i = sum_l W_{|i-l|} v_l, then adds Re(conj(v_i) s_i).  Per-tile partials are summed
 // in a fixed order by a second kernel, so the result is bitwise reproducible.
+#include <cooperative_groups.h>
+
 #include <mutex>
+#include <vector>
 
 #include "kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
 constexpr int QT = 128;
+constexpr int NOALLOC_MAX_DEVICES = 64;
 
 __device__ __forceinline__ void tile_of(int64_t b, int64_t& bi, int64_t& bl) {
   int64_t r = (int64_t)((sqrt(8.0 * (double)b + 1.0) - 1.0) * 0.5);
@@ -21,36 +27,43 @@ __device__ __forceinline__ void tile_of(int64_t b, int64_t& bi, int64_t& bl) {
   bl = b - r * (r + 1) / 2;
 }
 
+// A cluster of C blocks takes one tile, QT / C of its columns each, and adds the blocks' sums in
+// order through distributed shared memory: one partial per tile whatever C is.
+template <int C>
 __global__ void __launch_bounds__(QT)
 qform_tile_kernel(const double2* __restrict__ v, const double* __restrict__ lags, int64_t n,
                   double* __restrict__ partials) {
-  __shared__ double2 vl[QT];
-  __shared__ double lw[2 * QT];
+  constexpr int U = QT / C;
+  __shared__ double2 vl[U];
+  __shared__ double lw[QT + U];
   __shared__ double red[QT];
+  __shared__ double share[C];
+  const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;
+  const int64_t tile = blockIdx.x / C;
   int64_t bi, bl;
-  tile_of(blockIdx.x, bi, bl);
+  tile_of(tile, bi, bl);
   int t = threadIdx.x;
   int64_t i = bi * QT + t;
-  int64_t l0 = bl * QT;
-  int64_t base = (bi - bl) * QT;  // i - l = base + (t - u)
-  vl[t] = (l0 + t < n) ? v[l0 + t] : mkc(0.0, 0.0);
-  for (int d = t; d < 2 * QT - 1; d += QT) {
-    int64_t lag = base + d - (QT - 1);
+  int64_t l0 = bl * QT + rank * U;
+  int64_t base = bi * QT - l0;  // i - l = base + (t - u)
+  if (t < U) vl[t] = (l0 + t < n) ? v[l0 + t] : mkc(0.0, 0.0);
+  for (int d = t; d < QT + U - 1; d += QT) {
+    int64_t lag = base + d - (U - 1);
     if (lag < 0) lag = -lag;
     lw[d] = lag < n ? lags[lag] : 0.0;
   }
+  const double2 vi = i < n ? v[i] : mkc(0.0, 0.0);
   __syncthreads();
   double c = 0.0;
   if (i < n) {
     double sr = 0.0, si = 0.0;
 #pragma unroll 8
-    for (int u = 0; u < QT; ++u) {
-      double wv = lw[t - u + QT - 1];
+    for (int u = 0; u < U; ++u) {
+      double wv = lw[t - u + U - 1];
       double2 x = vl[u];
       sr = fma(wv, x.x, sr);
       si = fma(wv, x.y, si);
     }
-    double2 vi = v[i];
     c = vi.x * sr + vi.y * si;
   }
   red[t] = c;
@@ -59,7 +72,17 @@ qform_tile_kernel(const double2* __restrict__ v, const double* __restrict__ lags
     if (t < s) red[t] += red[t + s];
     __syncthreads();
   }
-  if (t == 0) partials[blockIdx.x] = (bi == bl ? 1.0 : 2.0) * red[0];
+  if constexpr (C > 1) {
+    cg::cluster_group cl = cg::this_cluster();
+    if (t == 0) cl.map_shared_rank(share, 0)[rank] = red[0];
+    cl.sync();
+    if (rank != 0 || t != 0) return;
+    double a = 0.0;
+    for (int r = 0; r < C; ++r) a += share[r];
+    partials[tile] = (bi == bl ? 1.0 : 2.0) * a;
+  } else {
+    if (t == 0) partials[tile] = (bi == bl ? 1.0 : 2.0) * red[0];
+  }
 }
 
 __global__ void __launch_bounds__(256)
@@ -76,6 +99,11 @@ sum_partials_kernel(const double* __restrict__ p, int64_t np, double* __restrict
   if (threadIdx.x == 0) *out = s[0];
 }
 
+constexpr int64_t QWS_TILES = 256 * 257 / 2;  // n <= 32768
+constexpr size_t QWS_KEEP = 8;
+std::mutex g_qws_mu;
+std::vector<QformWs> g_qws[NOALLOC_MAX_DEVICES];
+
 }  // namespace
 
 int64_t qform_num_partials(int64_t n) {
@@ -88,10 +116,72 @@ cudaError_t launch_qform(const double2* v, const double* lags, int64_t n, double
   if (n <= 0) return cudaErrorInvalidValue;
   int64_t np = qform_num_partials(n);
   if (np > 0x7fffffffLL) return cudaErrorInvalidValue;
-  qform_tile_kernel<<<(unsigned)np, QT, 0, s>>>(v, lags, n, partials); rci_note_launch();
+  // One tile keeps an SM's FP64 pipe busy for 9.4 us.  While the tiles are no more than the SMs
+  // (n <= 2176) eight blocks share each, so that the work spreads over the GPU: at n = 400 (ten
+  // tiles) 13.6 -> 7.3 us; beyond, one block per tile fills it.
+  if (np <= 153) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)np * 8);
+    cfg.blockDim = dim3(QT);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 8;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    RCI_CUDA_TRY(cudaLaunchKernelEx(&cfg, qform_tile_kernel<8>, v, lags, n, partials));
+  } else {
+    qform_tile_kernel<1><<<(unsigned)np, QT, 0, s>>>(v, lags, n, partials);
+  }
+  rci_note_launch();
   RCI_CUDA_TRY(cudaGetLastError());
   sum_partials_kernel<<<1, 256, 0, s>>>(partials, np, out_dev); rci_note_launch();
   return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- kept workspaces
+// rci_qform_toeplitz borrows its workspace (partials on the device, the result in pinned host
+// memory that the last kernel writes) for the length of a call and has waited for its stream when
+// it gives it back, so a workspace is never in use by two calls, whatever their threads and
+// streams.  cudaMalloc and cudaFree cost 0.17 ms a call, and the latter waits for the whole
+// device.  At most QWS_KEEP workspaces of QWS_TILES partials (257 KB, n <= 32768) are kept per
+// device; a call that finds none free allocates one, and it is released where enough are kept
+// already or it is larger.
+cudaError_t qform_borrow(QformWs* w, int64_t n) {
+  *w = QformWs{};
+  RCI_CUDA_TRY(cudaGetDevice(&w->device));
+  const int64_t np = qform_num_partials(n);
+  if (np <= QWS_TILES && w->device < NOALLOC_MAX_DEVICES) {
+    std::lock_guard<std::mutex> lk(g_qws_mu);
+    std::vector<QformWs>& v = g_qws[w->device];
+    if (!v.empty()) {
+      *w = v.back();
+      v.pop_back();
+      return cudaSuccess;
+    }
+  }
+  w->kept = np <= QWS_TILES && w->device < NOALLOC_MAX_DEVICES;
+  cudaError_t e = cudaMalloc(&w->part, sizeof(double) * (size_t)(w->kept ? QWS_TILES : np));
+  if (e == cudaSuccess) e = cudaHostAlloc(&w->result, sizeof(double), cudaHostAllocDefault);
+  if (e != cudaSuccess) {
+    cudaFree(w->part);
+    *w = QformWs{};
+  }
+  return e;
+}
+
+void qform_return(const QformWs& w, bool ok) {
+  if (w.kept && ok) {
+    std::lock_guard<std::mutex> lk(g_qws_mu);
+    std::vector<QformWs>& v = g_qws[w.device];
+    if (v.size() < QWS_KEEP) {
+      v.push_back(w);
+      return;
+    }
+  }
+  cudaFree(w.part);
+  cudaFreeHost(w.result);
 }
 
 // ---------------------------------------------------------------- allocation-free variant
@@ -109,7 +199,6 @@ cudaError_t launch_qform(const double2* v, const double* lags, int64_t n, double
 namespace {
 constexpr int64_t NOALLOC_TILES = RCI_QFORM_NOALLOC_MAX_N / QT;                // 256
 constexpr int64_t NOALLOC_PARTIALS = NOALLOC_TILES * (NOALLOC_TILES + 1) / 2;  // 32896
-constexpr int NOALLOC_MAX_DEVICES = 64;
 static_assert(RCI_QFORM_NOALLOC_MAX_N % QT == 0, "maximum size must be a whole number of tiles");
 }  // namespace
 
