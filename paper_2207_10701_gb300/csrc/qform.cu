@@ -118,7 +118,7 @@ cudaError_t launch_qform(const double2* v, const double* lags, int64_t n, double
   if (np > 0x7fffffffLL) return cudaErrorInvalidValue;
   // One tile keeps an SM's FP64 pipe busy for 9.4 us.  While the tiles are no more than the SMs
   // (n <= 2176) eight blocks share each, so that the work spreads over the GPU: at n = 400 (ten
-  // tiles) 13.6 -> 7.3 us; beyond, one block per tile fills it.
+  // tiles) 13.6 -> 7.0 us; beyond, one block per tile fills it.
   if (np <= 153) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)np * 8);

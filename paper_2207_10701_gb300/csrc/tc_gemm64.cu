@@ -13,10 +13,11 @@
 // 5 to 7 share an accumulator and 5.8e-16 without i + j = 7.  Per output the accumulators are
 // joined in 64-bit integers and rounded once to FP64.
 //
-// Measured, 608 products of 160^3: SG_FULL 897 us (1.48 us a product, 22 TFLOP/s of FP64 work;
-// the FP64 GEMM takes 28 us a product), SG_HALF 459 us; splitting an operand 0.25 us.  Bound by the
-// MMAs' reading of the A operand from shared memory (50 cycles each at N = 64, where the tensor
-// cores need 32) and by the epilogue (about a third).
+// Measured, 608 products of 160^3: SG_FULL 710 us (1.17 us a product, 28 TFLOP/s of FP64 work; the
+// FP64 GEMM takes 28 us a product; 897 us with A in shared memory and an epilogue that the MMAs
+// wait for), SG_HALF 463 us; splitting an operand 0.25 us.  Bound by the MMAs (47 cycles each at
+// N = 64 with the copies of A, where the tensor cores need 32) and by the joining of the
+// accumulators (about a fifth).
 //
 // Layout.  A split form holds, per 16 terms k and digit s, planes r, i and -r of bf16 core
 // matrices (8 rows x 8 terms, 128 bytes), so every shared-memory operand is a run of contiguous
@@ -27,8 +28,10 @@
 // Roles of a persistent CTA (one per SM, 18 warps): warp 0 copies (stages of 16 terms, all
 // digits), warp 1 issues a stage's MMAs (one wait per stage: a wait per digit made the loop
 // twice as long), warps 2-17 join the accumulators, transpose through shared memory and store
-// whole 256-byte row pieces.  The accumulators fill the tensor memory, so an epilogue is not
-// hidden under the next tile's MMAs, but the stages fill meanwhile.
+// whole 256-byte row pieces.  The accumulators fill the tensor memory, so the next tile's MMAs
+// start when they have been joined into registers, under the stores.  SG_FULL copies a digit's A
+// windows to tensor memory once for all its pairs (tcgen05.cp): with A in shared memory an MMA
+// of 64 columns is bound by reading it.
 #include "tc_gemm64.cuh"
 #include "tc_gemm.cuh"
 
@@ -55,6 +58,8 @@ struct SgCfg {
   static constexpr int STAGES = 3 * STAGE + 2 * SG_STG_BYTES + 128 <= SG_SMEM_MAX ? 3 : 2;
   static constexpr uint32_t STG_OFF = STAGES * STAGE;
   static constexpr uint32_t BAR_OFF = STG_OFF + 2 * SG_STG_BYTES;
+  // A operands copied to tensor memory beside the accumulators where those leave four pairs of slots
+  static constexpr bool TS = 512 - ACC * NT >= 64;
   static constexpr uint32_t SMEM = BAR_OFF + (2 * STAGES + 3) * 8 + 16;
   static_assert(SMEM <= SG_SMEM_MAX, "one CTA per SM beside the static shared memory");
   static_assert(SLOT % 128 == 0 && STG_OFF % 16 == 0 && NT % 16 == 0 && ACC * NT <= 512, "layout");
@@ -65,7 +70,7 @@ constexpr long long SG_OWN_WAIT = 4000000000LL;
 
 struct SgArgs {
   int M, N, K;
-  int nt, ntiles_n, ntiles_m, chunks;  // columns per tile, tiles, 16-term chunks
+  int nt, ntiles_n, ntiles_m, chunks;  // columns per tile (the last one narrower), tiles, 16-term chunks
   int GA, GB;                          // 8-row groups of the A and B forms
   int njob, ntiles;
   int tile0[2];
@@ -134,6 +139,20 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint32_t hi, uint32_t a, ui
       " mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
       " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(d),
       "r"(a), "r"(b), "r"(idesc), "r"(hi), "r"(acc));
+}
+// the same with A in tensor memory (128 lanes x 8 columns)
+__device__ __forceinline__ void mma_bf16_t(uint32_t d, uint32_t hi, uint32_t a, uint32_t b, uint32_t idesc,
+                                           uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 db;\n setp.ne.b32 p, %5, 0;\n mov.b64 db, {%2, %4};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n}\n" ::"r"(d),
+      "r"(a), "r"(b), "r"(idesc), "r"(hi), "r"(acc));
+}
+// 128 rows x 16 terms from shared memory (descriptor lo, hi) to tensor memory
+__device__ __forceinline__ void copy_a(uint32_t t, uint32_t lo, uint32_t hi) {
+  asm volatile("{\n .reg .b64 da;\n mov.b64 da, {%1, %2};\n tcgen05.cp.cta_group::1.128x256b [%0], da;\n}\n" ::"r"(t),
+               "r"(lo), "r"(hi)
+               : "memory");
 }
 __device__ __forceinline__ void commit(uint64_t* b) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s32(b))
@@ -217,7 +236,7 @@ __device__ __forceinline__ void f_after() { asm volatile("tcgen05.fence::after_t
 // part in, every pass a full accumulation and epilogue of its own (the segments' operands have
 // their own exponents).
 struct Tile {
-  int j, z, i0, n0;
+  int j, z, i0, n0, nt;  // nt: the tile's columns rounded up to 16
   bool run, v[2];
 };
 __device__ __forceinline__ Tile tile_at(const SgJob* jobs, const SgArgs& p, int t) {
@@ -230,6 +249,7 @@ __device__ __forceinline__ Tile tile_at(const SgJob* jobs, const SgArgs& p, int 
   const int im = q / p.ntiles_n;
   r.i0 = im * SG_ROWS;
   r.n0 = (q - im * p.ntiles_n) * p.nt;
+  r.nt = min(p.nt, (p.N - r.n0 + 15) & ~15);
   const SgJob& jb = jobs[r.j];
   r.run = jb.skip == nullptr || jb.skip[r.z] == 0;
   r.v[0] = r.run && r.z >= jb.seg[0].zlo && r.z < jb.seg[0].zhi;
@@ -253,6 +273,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
   __shared__ SgJob jobs[2];
   __shared__ int32_t sh_eb[SG_NT];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (p.njob == 1 && p.job[0].any && *p.job[0].any == 0) return;
   if (tid == 0) {
     jobs[0] = p.job[0];
     jobs[1] = p.job[1];
@@ -289,7 +310,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
         const SgSeg& sg = jobs[tl.j].seg[g];
         const int ga0 = tl.i0 >> 3, gb0 = tl.n0 >> 3;
         const uint32_t ba = 256u * (uint32_t)min(SG_ROWS / 8, p.GA - ga0);
-        const uint32_t bb = 256u * (uint32_t)min(p.nt / 8, p.GB - gb0);
+        const uint32_t bb = 256u * (uint32_t)min(tl.nt / 8, p.GB - gb0);
         const int64_t fa = (int64_t)p.chunks * SG_SLICES * sg.planesA * p.GA * 256;
         const int64_t fb = (int64_t)p.chunks * SG_SLICES * sg.planesB * p.GB * 256;
         const unsigned char* A = sg.A + (tl.z + sg.zA) * fa + ga0 * 256;
@@ -333,9 +354,6 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issue
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.nt >> 3) << 17) |
-                           ((uint32_t)(128 >> 4) << 24);
-    const uint32_t ineg = idesc | (1u << 13);  // -A
     const uint32_t ntu = (uint32_t)p.nt;
     const uint32_t dlo = (SG_LBO >> 4) << 16, dhi = (SG_SBO >> 4) | (1u << 14);
     constexpr uint32_t SLOT16 = SG_SLOT >> 4, A16 = SG_A_SLOT >> 4, R16 = (SG_ROWS * 32) >> 4, B16 = SG_B_PLANE >> 4;
@@ -350,6 +368,9 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
           break;
         }
         f_after();
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tl.nt >> 3) << 17) |
+                               ((uint32_t)(128 >> 4) << 24);
+        const uint32_t ineg = idesc | (1u << 13);  // -A
         for (int c = 0; c < p.chunks; ++c, ++it) {
           const int st = it % SG_STAGES;
           if (!wait_warp(&full[st], (uint32_t)((it / SG_STAGES) & 1), abort_flag, p.wait_limit)) {
@@ -361,13 +382,26 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
             const uint32_t more = c > 0 ? 1u : 0u;  // the first pair of an accumulator overwrites it
 #pragma unroll
             for (int i = 0; i < Cfg::DIG; ++i) {
+              // both windows of the digit, read once from shared memory for all its pairs (copies
+              // and MMAs of one thread run in order, so a slot is free when its turn comes again)
+              const uint32_t ta = tmem + (uint32_t)(SG_ACC * SG_NT) + 16u * (uint32_t)(i & 3);
+              if (Cfg::TS) {
+                copy_a(ta, a0 + i * SLOT16, dhi);
+                copy_a(ta + 8u, a0 + R16 + i * SLOT16, dhi);
+              }
 #pragma unroll
               for (int j = 0; j < Cfg::DIG; ++j) {
                 if (i + j >= Cfg::W) continue;
                 const int w = i + j < SG_ACC - 1 ? i + j : SG_ACC - 1;
                 const uint32_t d = tmem + (uint32_t)w * ntu;
-                mma_bf16(d, dhi, a0 + i * SLOT16, b0 + j * SLOT16, idesc, i == 0 && j < SG_ACC ? more : 1u);
-                mma_bf16(d, dhi, a0 + R16 + i * SLOT16, b0 + B16 + j * SLOT16, ineg, 1u);
+                const uint32_t on = i == 0 && j < SG_ACC ? more : 1u;
+                if (Cfg::TS) {
+                  mma_bf16_t(d, dhi, ta, b0 + j * SLOT16, idesc, on);
+                  mma_bf16_t(d, dhi, ta + 8u, b0 + B16 + j * SLOT16, ineg, 1u);
+                } else {
+                  mma_bf16(d, dhi, a0 + i * SLOT16, b0 + j * SLOT16, idesc, on);
+                  mma_bf16(d, dhi, a0 + R16 + i * SLOT16, b0 + B16 + j * SLOT16, ineg, 1u);
+                }
               }
             }
             commit(&empty[st]);
@@ -418,18 +452,14 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
         ok = agree(wait_warp(acc_full, (uint32_t)(ps & 1), abort_flag, p.wait_limit));
         if (!ok) break;
         f_after();
-        const int last = min(p.nt >> 4, (p.N - tl.n0 + 15) >> 4);
-        for (int sb = 0; sb < last; ++sb) {
-          // this thread's outputs of the slab, rows r and r + 32, column col; their C0 first
-          const int col = tl.n0 + 16 * sb + (et & 15);
-          const int r = et >> 4;
-          double2 c0[2];
+        // join the accumulators of all the tile's slabs into registers, so that the next tile's MMAs
+        // start while the results are stored
+        constexpr int SLABS = SG_NT / 16;
+        const int last = tl.nt >> 4;
+        double v[SLABS][4];
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int gr = tl.i0 + r + 32 * i;
-            c0[i] = (C0 && gr < p.M && col < p.N) ? C0[(int64_t)gr * ldc0 + col] : make_double2(0.0, 0.0);
-            if (eye && gr == col) c0[i].x = 1.0;
-          }
+        for (int sb = 0; sb < SLABS; ++sb) {
+          if (sb >= last) break;
           float a[SG_ACC][4];
 #pragma unroll
           for (int w = 0; w < SG_ACC; ++w) tmem_ld4(tl_base + (uint32_t)(w * p.nt + 16 * sb + c4), a[w]);
@@ -439,8 +469,6 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
             __syncwarp();
             if (lane == 0) bar_arrive(acc_empty);
           }
-          double* sp = reinterpret_cast<double*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES) +
-                       (row * SG_STG_LD + c4) * 2 + part;
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             // accumulator w in units of 2^(-8 w), joined in units of 2^(-8 (ACC - 1))
@@ -453,8 +481,26 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
               else lo += n;
               u *= 256.f;
             }
-            sp[2 * j] = scaled<8 * (SG_ACC > 3 ? SG_ACC - 3 : 0)>(hi, lo, ea, sh_eb[16 * sb + c4 + j]);
+            v[sb][j] = scaled<8 * (SG_ACC > 3 ? SG_ACC - 3 : 0)>(hi, lo, ea, sh_eb[16 * sb + c4 + j]);
           }
+        }
+#pragma unroll
+        for (int sb = 0; sb < SLABS; ++sb) {
+          if (sb >= last) break;
+          // this thread's outputs of the slab, rows r and r + 32, column col; their C0 first
+          const int col = tl.n0 + 16 * sb + (et & 15);
+          const int r = et >> 4;
+          double2 c0[2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int gr = tl.i0 + r + 32 * i;
+            c0[i] = (C0 && gr < p.M && col < p.N) ? C0[(int64_t)gr * ldc0 + col] : make_double2(0.0, 0.0);
+            if (eye && gr == col) c0[i].x = 1.0;
+          }
+          double* sp = reinterpret_cast<double*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES) +
+                       (row * SG_STG_LD + c4) * 2 + part;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sp[2 * j] = v[sb][j];
           // the slab is whole; the other buffer's slab has been read by every warp before this
           asm volatile("bar.sync 1, %0;" ::"n"(32 * SG_EPI_WARPS) : "memory");
           const double2* sr = reinterpret_cast<const double2*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES);
@@ -662,8 +708,12 @@ cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t strid
 namespace {
 template <typename Cfg>
 cudaError_t launch_cfg(SgArgs& a, int64_t products, cudaStream_t s) {
+  // Columns of a tile.  With A in tensor memory an MMA's time grows with its columns (33 cycles for
+  // 32, 47 for 64): full tiles and a narrower last one.  With A in shared memory it hardly does (48
+  // for 32, 58 for 96): equal tiles.  Narrow ones where even they do not fill the GPU.
   a.ntiles_n = (int)ceil_div(a.N, Cfg::NT);
-  a.nt = (int)ceil_div(ceil_div(a.N, a.ntiles_n), 16) * 16;  // equal column tiles
+  a.nt = Cfg::TS ? Cfg::NT : (int)ceil_div(ceil_div(a.N, a.ntiles_n), 16) * 16;
+  if (products * a.ntiles_m * ceil_div(a.N, 32) <= sm_count()) a.nt = 32;
   a.ntiles_n = (int)ceil_div(a.N, a.nt);
   const int64_t per = (int64_t)a.ntiles_m * a.ntiles_n, nt = products * per;
   if (nt > 0x7fffffffLL) return cudaErrorInvalidValue;

@@ -36,7 +36,8 @@ struct SgSeg {
 // C may be C0).  Every output takes part in at least one segment.  identity: C0 is the identity
 // matrix.  maxabs[z] (or null): atomicMax of the bits of the largest |re|, |im| of output z as a
 // float (rounded up by less than 2^-20; infinity for anything not finite).
-// Products with skip[z] != 0 (or null) are left out, C[z] untouched.
+// Products with skip[z] != 0 (or null) are left out, C[z] untouched; *any == 0 (or null) says that
+// all of a one-job launch are.
 struct SgJob {
   int nseg;
   SgSeg seg[2];
@@ -48,6 +49,7 @@ struct SgJob {
   int batch;
   uint32_t* maxabs;
   const int32_t* skip;
+  const int32_t* any;
 };
 
 // Digit pairs kept: SG_FULL the 34 that count in FP64 (error about 2^-55 of the product of the
