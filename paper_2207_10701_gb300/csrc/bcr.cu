@@ -1997,15 +1997,15 @@ cudaError_t bcr_read_status(BcrHandle* h, int32_t* st, cudaStream_t s, double* g
 // ===================================================================== FP64 on the tensor cores
 // The FP64 factorisation runs its block products through the digit split of tc_gemm64.cu and its
 // block inverses as Newton iterations on an FP32 inverse, X <- X + X (I - D X), with those products:
-// the FP64 pipe does neither.  At ny = 160 a product takes 1.5 us of the whole GPU where the FP64
+// the FP64 pipe does neither.  At ny = 160 a product takes 1.2 us of the whole GPU where the FP64
 // GEMM took 28, and an inverse of one block alone 0.4 ms where the FP64 Gauss-Jordan took 4.9: a
-// new design of 500 cells 404 -> 49 ms, of 50 cells (ny = 128) 54 -> 10.3 ms.
+// new design of 500 cells 404 -> 42 ms, of 50 cells (ny = 128) 54 -> 6.7 ms.
 // A block whose iteration does not contract (an FP32 inverse that resolves nothing, entries outside
 // the FP32 range, a singular block) goes to the FP64 Gauss-Jordan kernel, which also reports zero
 // pivots, so the factorisation accepts and refuses what it did.
 //
-// Scratch: the handle's (m0 blocks of ny x ny); the blocks of a level are taken in batches that
-// fit it.
+// Scratch: the handle's (m0 blocks of ny x ny) and whatever of its working arrays and store the
+// step at hand leaves unused; the blocks of a level are taken in batches that fit it.
 namespace {
 
 // a = (float) of `batch` nn-element blocks, stride elements apart
@@ -2034,6 +2034,7 @@ struct NewtonFlags {
   int32_t* skip_r;    // no further residual wanted
   int32_t* skip_x;    // no further update wanted
   int32_t* failed;
+  int32_t* active;    // blocks whose update of this step, and whose next residual, are wanted
 };
 __global__ void newton_check_kernel(NewtonFlags f, int n, int batch, int rough, int last,
                                     const int32_t* __restrict__ st32, int32_t* status) {
@@ -2049,72 +2050,129 @@ __global__ void newton_check_kernel(NewtonFlags f, int n, int batch, int rough, 
   const bool contracts = m * (float)n < 0.25f;
   const bool done = contracts && !rough && (float)n * m * m <= 1e-17f;
   if (!contracts || (last && !done)) f.failed[z] = f.skip_x[z] = 1;
+  else atomicAdd(&f.active[0], 1);
   if (!contracts || done || last) f.skip_r[z] = 1;
+  else atomicAdd(&f.active[1], 1);
 }
 
 constexpr int NEWTON_STEPS = 4;
 
-// scratch of `bytes` at `base`, carved in 256-byte units
-struct Carve {
-  unsigned char* p;
+// Scratch memory in a few regions, handed out in 256-byte units from the region with most left.
+struct Scratch {
+  struct Region {
+    unsigned char* p;
+    size_t bytes, used;
+  };
+  std::vector<Region> r;
+  bool full = false;
+  void add(void* p, int64_t bytes) {
+    if (bytes > 0) r.push_back(Region{(unsigned char*)p, (size_t)bytes, 0});
+  }
+  void reset() {
+    for (Region& g : r) g.used = 0;
+    full = false;
+  }
   template <typename P> P* take(size_t bytes) {
-    P* r = reinterpret_cast<P*>(p);
-    p += (bytes + 255) & ~(size_t)255;
-    return r;
+    bytes = (bytes + 255) & ~(size_t)255;
+    Region* best = nullptr;
+    for (Region& g : r)
+      if (g.bytes - g.used >= bytes && (!best || g.bytes - g.used > best->bytes - best->used)) best = &g;
+    if (!best) {
+      full = true;
+      return nullptr;
+    }
+    unsigned char* q = best->p + best->used;
+    best->used += bytes;
+    return reinterpret_cast<P*>(q);
   }
 };
-inline size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// bytes per block of a batch: the Newton iteration, and the products of a reduction level
-size_t newton_block_bytes(int ny) {
-  const size_t nn = (size_t)ny * ny;
-  return 2 * up256(nn * 8) + up256(nn * 16) + 2 * sg_form_bytes(ny, ny, 3) + 2 * sg_form_bytes(ny, ny, 2) +
-         5 * 256 + 4 * up256(sizeof(int32_t) * sg_form_exps(ny));
-}
-size_t level_block_bytes(int ny) {
-  return 3 * sg_form_bytes(ny, ny, 3) + 2 * sg_form_bytes(ny, ny, 2) +
-         5 * up256(sizeof(int32_t) * sg_form_exps(ny));
+// A split form and its exponents, for up to c operands.
+struct Form {
+  unsigned char* f;
+  int32_t* e;
+  Form() = default;
+  Form(Scratch& w, int rows, int K, int planes, size_t c)
+      : f(w.take<unsigned char>(c * sg_form_bytes(rows, K, planes))),
+        e(w.take<int32_t>(4 * c * (size_t)sg_form_exps(rows))) {}
+};
+
+// The buffers of one batch of c blocks.  (A region's alignment is that of device allocations or of
+// whole blocks: a multiple of 16 bytes, what the copies need.)
+struct NewtonBuf {
+  Form D, Xr, C;      // D and X as left operands; the right one in turn, X or R
+  double2* R;         // first the FP32 copies of D and X
+  int32_t* words;
+  NewtonBuf(Scratch& w, int ny, size_t c) {
+    D = Form(w, ny, ny, 3, c);
+    Xr = Form(w, ny, ny, 3, c);
+    C = Form(w, ny, ny, 2, c);
+    R = w.take<double2>(c * ny * ny * sizeof(double2));
+    words = w.take<int32_t>(4 * (4 * c + 1 + 2 * NEWTON_STEPS));
+  }
+};
+struct LevelBuf {
+  Form D, O, E, X, Y;
+  LevelBuf(Scratch& w, int ny, size_t c) {
+    D = Form(w, ny, ny, 3, c + 1);  // Dinv; once X and Y are formed, the columns of X
+    X = D;
+    O = Form(w, ny, ny, 3, c);
+    E = Form(w, ny, ny, 3, c + 1);
+    Y = Form(w, ny, ny, 2, c + 1);
+  }
+};
+struct FwdBuf {
+  Form D, X, Y, B;
+  FwdBuf(Scratch& w, int ny, int nq, size_t c) {
+    D = Form(w, ny, ny, 3, c);
+    X = Form(w, ny, ny, 3, c);
+    Y = Form(w, ny, ny, 3, c + 1);
+    B = Form(w, nq, ny, 2, c + 1);
+  }
+};
+
+// the most blocks (at most `want`) whose buffers fit, so that the batches are equal; 0: none
+template <typename Place>
+int batch_of(Scratch& w, int want, Place place) {
+  auto fits = [&](int c) {
+    w.reset();
+    place(c);
+    return !w.full;
+  };
+  int lo = 0, hi = std::min(want, 32768);
+  if (want < 1) return 0;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) / 2;
+    if (fits(mid)) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo == 0 ? 0 : (int)ceil_div(want, ceil_div(want, lo));
 }
 
 }  // namespace
 
-// blocks per batch that `bytes` of scratch hold (0: the FP64 split path does not apply)
-static int split_batch(int ny, size_t bytes) {
-  if (ny > SG_KMAX) return 0;
-  const size_t per = std::max(newton_block_bytes(ny), level_block_bytes(ny));
-  const size_t fixed = 3 * level_block_bytes(ny) + 16 * 256;  // the levels' one extra block per form
-  return bytes <= fixed ? 0 : (int)std::min<size_t>((bytes - fixed) / per, 4096);
-}
-
 // out[z] = D[z]^-1 for z < m (D: stride elements apart, destroyed where the Gauss-Jordan kernel
 // takes over).
-static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int ny, int m, int cmax,
-                                 void* scratch, int32_t* status, cudaStream_t s) {
+static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int ny, int m, Scratch& mem,
+                                 int32_t* status, cudaStream_t s) {
   const int64_t nn = (int64_t)ny * ny;
-  const int nb = (int)ceil_div(m, cmax), cb = (int)ceil_div(m, nb);
+  const int cb = batch_of(mem, m, [&](int c) { NewtonBuf(mem, ny, c); });
+  if (cb == 0) return cudaErrorInvalidValue;
   const long long wl = tc_wait_limit();
   for (int k0 = 0; k0 < m; k0 += cb) {
     const int c = std::min(cb, m - k0);
-    Carve w{(unsigned char*)scratch};
-    float2* a32 = w.take<float2>((size_t)c * nn * 8);
-    float2* x32 = w.take<float2>((size_t)c * nn * 8);
-    double2* R = w.take<double2>((size_t)c * nn * 16);
-    const size_t f3 = sg_form_bytes(ny, ny, 3), f2 = sg_form_bytes(ny, ny, 2);
-    const int ne = sg_form_exps(ny);
-    unsigned char* fD = w.take<unsigned char>(c * f3);
-    unsigned char* fXr = w.take<unsigned char>(c * f3);
-    unsigned char* fXc = w.take<unsigned char>(c * f2);
-    unsigned char* fR = w.take<unsigned char>(c * f2);
-    int32_t* eD = w.take<int32_t>(sizeof(int32_t) * ne * c);
-    int32_t* eXr = w.take<int32_t>(sizeof(int32_t) * ne * c);
-    int32_t* eXc = w.take<int32_t>(sizeof(int32_t) * ne * c);
-    int32_t* eR = w.take<int32_t>(sizeof(int32_t) * ne * c);
-    int32_t* words = w.take<int32_t>(sizeof(int32_t) * (4 * (size_t)c + 1));
-    const NewtonFlags fl{reinterpret_cast<uint32_t*>(words), words + c, words + 2 * c, words + 3 * c};
+    mem.reset();
+    const NewtonBuf w(mem, ny, c);
+    float2* a32 = reinterpret_cast<float2*>(w.R);
+    float2* x32 = a32 + c * nn;
+    double2* R = w.R;
+    unsigned char *fD = w.D.f, *fXr = w.Xr.f, *fXc = w.C.f, *fR = w.C.f;
+    int32_t *eD = w.D.e, *eXr = w.Xr.e, *eXc = w.C.e, *eR = w.C.e;
+    int32_t* words = w.words;
     int32_t* st32 = words + 4 * c;
     double2* Dk = D + (int64_t)k0 * stride;
     double2* X = out + (int64_t)k0 * nn;
-    RCI_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(int32_t) * (4 * (size_t)c + 1), s));
+    RCI_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(int32_t) * (4 * (size_t)c + 1 + 2 * NEWTON_STEPS), s));
     const int64_t tot = (int64_t)c * nn;
     blocks_to_f32_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(Dk, stride, nn, tot, a32);
     rci_note_launch();
@@ -2126,6 +2184,8 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
     RCI_CUDA_TRY(cudaGetLastError());
     RCI_CUDA_TRY(launch_sg_split(Dk, false, ny, stride, false, ny, ny, 3, c, fD, eD, nullptr, s));
     for (int it = 0; it < NEWTON_STEPS; ++it) {
+      const NewtonFlags fl{reinterpret_cast<uint32_t*>(words), words + c, words + 2 * c, words + 3 * c,
+                           st32 + 1 + 2 * it};
       RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, true, ny, ny, 2, c, fXc, eXc, fl.skip_r, s));
       SgJob r{};
       r.nseg = 1;
@@ -2138,6 +2198,7 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
       r.batch = c;
       r.maxabs = fl.maxabs;
       r.skip = fl.skip_r;
+      if (it > 0) r.any = st32 + 2 * it;  // what the step before left active
       RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &r, it == 0 ? SG_HALF : SG_FULL, status, wl, s));
       newton_check_kernel<<<(unsigned)ceil_div(c, 128), 128, 0, s>>>(fl, ny, c, it == 0, it == NEWTON_STEPS - 1,
                                                                      st32, status);
@@ -2156,9 +2217,10 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
       x.sC = nn;
       x.batch = c;
       x.skip = fl.skip_x;
+      x.any = &fl.active[0];
       RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &x, SG_HALF, status, wl, s));
     }
-    RCI_CUDA_TRY(launch_gj_simt<double>(Dk, stride, X, nn, ny, c, status, s, fl.failed));
+    RCI_CUDA_TRY(launch_gj_simt<double>(Dk, stride, X, nn, ny, c, status, s, words + 3 * c));
   }
   return cudaSuccess;
 }
@@ -2171,30 +2233,24 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
 // and the left one of D', the rows of L_{2k} as the right operand of Y (of the row before) and the
 // left one of D' and L'.
 static cudaError_t split_level(const double2* D, const double2* L, const double2* Dinv, double2* X, double2* Y,
-                               double2* Dn, double2* Ln, int ny, int n, int m, int nk, int cmax, void* scratch,
+                               double2* Dn, double2* Ln, int ny, int n, int m, int nk, Scratch& mem,
                                int32_t* status, Profiler* prof, cudaStream_t s) {
   const int64_t nn = (int64_t)ny * ny;
   const int my = (n - 1) / 2;
-  const int nb = (int)ceil_div(nk, cmax), cb = (int)ceil_div(nk, nb);
-  const size_t f3 = sg_form_bytes(ny, ny, 3), f2 = sg_form_bytes(ny, ny, 2);
+  const size_t f3 = sg_form_bytes(ny, ny, 3);
   const int ne = sg_form_exps(ny);
+  const int cb = batch_of(mem, nk, [&](int c) { LevelBuf(mem, ny, c); });
+  if (cb == 0) return cudaErrorInvalidValue;
   const long long wl = tc_wait_limit();
   for (int k0 = 0; k0 < nk; k0 += cb) {
     const int c = std::min(cb, nk - k0);           // kept rows k0 .. k0 + c - 1
     const int cm = std::min(c, m - k0);            // of which eliminated rows of the same index
     const int cy = std::max(0, std::min(c, my - k0));
     const int p0 = k0 > 0 ? 1 : 0;                 // X, Y of row k0 - 1 come first
-    Carve w{(unsigned char*)scratch};
-    unsigned char* fD = w.take<unsigned char>(c * f3);
-    unsigned char* fO = w.take<unsigned char>(c * f3);
-    unsigned char* fE = w.take<unsigned char>((c + 1) * f3);
-    unsigned char* fX = w.take<unsigned char>((c + 1) * f2);
-    unsigned char* fY = w.take<unsigned char>((c + 1) * f2);
-    int32_t* eD = w.take<int32_t>(sizeof(int32_t) * ne * c);
-    int32_t* eO = w.take<int32_t>(sizeof(int32_t) * ne * c);
-    int32_t* eE = w.take<int32_t>(sizeof(int32_t) * ne * (c + 1));
-    int32_t* eX = w.take<int32_t>(sizeof(int32_t) * ne * (c + 1));
-    int32_t* eY = w.take<int32_t>(sizeof(int32_t) * ne * (c + 1));
+    mem.reset();
+    const LevelBuf w(mem, ny, c);
+    unsigned char *fD = w.D.f, *fO = w.O.f, *fE = w.E.f, *fX = w.X.f, *fY = w.Y.f;
+    int32_t *eD = w.D.e, *eO = w.O.e, *eE = w.E.e, *eX = w.X.e, *eY = w.Y.e;
     // L_{2k} for k = k0 .. k0 + c while it exists (index 2k <= n - 1; L_0 is not used)
     const int nE = std::min(c + 1, nk - k0);
     const int pm = p0 + std::max(0, cm), py = p0 + cy;
@@ -2305,9 +2361,31 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
   int cur = 0;
   auto store = (cplx<T>*)h->store;
   // FP64 on the tensor cores where the scratch holds at least one block
-  int cmax = 0;
-  if constexpr (sizeof(T) == 8)
-    cmax = split_batch(ny, (size_t)std::max<int64_t>(m0, 1) * nn * sizeof(cplx<T>));
+  // the scratch of an inversion (sch == false) or of the products of level l
+  auto scratch_of = [&](int l, bool sch) {
+    Scratch w;
+    const int64_t bb = nn * (int64_t)sizeof(cplx<T>), nl = h->n[l], nk = l < h->Lf ? h->n[l + 1] : 0;
+    w.add(h->scratch, std::max<int64_t>(m0, 1) * bb);
+    for (void** a : {&h->Dw[0], &h->Lw[0]}) {
+      w.add((char*)a[cur] + nl * bb, (n1 - nl) * bb);
+      w.add((char*)a[1 - cur] + (sch ? nk * bb : 0), (n1 - (sch ? nk : 0)) * bb);
+    }
+    // the store of this level's products while its blocks are inverted, and of the levels to come
+    const int64_t from = l >= h->Lf ? h->final_off + nn : sch ? h->off[l + 1] : h->off[l] + h->m[l] * nn;
+    w.add((cplx<T>*)h->store + from, (h->final_off + nn - from) * (int64_t)sizeof(cplx<T>));
+    return w;
+  };
+  // (taken where the scratch of every step holds at least one block: a dozen columns or more)
+  bool split = sizeof(T) == 8 && ny <= SG_KMAX;
+  if constexpr (sizeof(T) == 8) {
+    for (int l = 1; l <= h->Lf && split; ++l) {
+      Scratch wi = scratch_of(l, false);
+      split = batch_of(wi, 1, [&](int c) { NewtonBuf(wi, ny, c); }) == 1;
+      if (l == h->Lf || !split) break;
+      Scratch ws = scratch_of(l, true);
+      split = batch_of(ws, 1, [&](int c) { LevelBuf(ws, ny, c); }) == 1;
+    }
+  }
   for (int l = 1; l < h->Lf; ++l) {
     const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
     const int my = (n - 1) / 2;
@@ -2322,12 +2400,13 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     {
       ProfScope ps(h->prof, PF_INVERT, s, 8.0 * ny * (double)nn * m, 2.0 * m * nn * sizeof(cplx<T>), 1);
       if constexpr (sizeof(T) == 8) {
-        if (cmax > 0) {
+        if (split) {
           RCI_CUDA_TRY(launch_block_maxabs<T>(D + nn, 2 * nn, nn, m, maxabs + 1, s));
-          RCI_CUDA_TRY(split_inverse(D + nn, 2 * nn, Dinv, ny, m, cmax, h->scratch, h->status, s));
+          Scratch w = scratch_of(l, false);
+          RCI_CUDA_TRY(split_inverse(D + nn, 2 * nn, Dinv, ny, m, w, h->status, s));
         }
       }
-      if (cmax == 0) RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
+      if (!split) RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
                                 !h->simt));
     }
     // X_k = Dinv_k L_{2k+1};  Y_k = Dinv_k L_{2k+2}^T
@@ -2337,8 +2416,9 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
     // over K = 2 ny (written once) together with L'; otherwise five batched products.
     bool fused = false;
     if constexpr (sizeof(T) == 8) {
-      if (cmax > 0) {
-        RCI_CUDA_TRY(split_level(D, L, Dinv, X, Y, Dn, Ln, ny, n, m, nk, cmax, h->scratch, h->status, h->prof, s));
+      if (split) {
+        Scratch w = scratch_of(l, true);
+        RCI_CUDA_TRY(split_level(D, L, Dinv, X, Y, Dn, Ln, ny, n, m, nk, w, h->status, h->prof, s));
         fused = true;
       }
     }
@@ -2413,9 +2493,10 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
   {
     ProfScope ps(h->prof, PF_INVERT, s, 8.0 * ny * (double)nn, 2.0 * nn * sizeof(cplx<T>), 1);
     if constexpr (sizeof(T) == 8) {
-      if (cmax > 0) {
+      if (split) {
         RCI_CUDA_TRY(launch_block_maxabs<T>((cplx<T>*)h->Dw[cur], nn, nn, 1, maxabs + 1, s));
-        return split_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, cmax, h->scratch, h->status, s);
+        Scratch w = scratch_of(h->Lf, false);
+        return split_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, w, h->status, s);
       }
     }
     RCI_CUDA_TRY(launch_gj<T>((cplx<T>*)h->Dw[cur], 0, store + h->final_off, 0, ny, 1, h->status, s,
@@ -2522,38 +2603,30 @@ static cudaError_t multi_update(BcrHandle* h, int ny, int nq, const MultiTerm<T>
   return cudaSuccess;
 }
 
-// blocks per batch of the FP64 split solve that the handle's scratch holds (0: not taken)
-static int split_solve_batch(const BcrHandle* h, int nq) {
-  const int ny = h->ny;
-  if (ny > SG_KMAX) return 0;
-  const size_t bytes = (size_t)std::max<int64_t>(h->m[0], 1) * ny * ny * sizeof(double2);
-  const size_t per = 3 * (sg_form_bytes(ny, ny, 3) + up256(4 * sg_form_exps(ny))) + sg_form_bytes(nq, ny, 2) +
-                     up256(4 * sg_form_exps(nq));
-  const size_t fixed = 2 * per + 16 * 256;  // one block more per form
-  return bytes <= fixed ? 0 : (int)std::min<size_t>((bytes - fixed) / per, 4096);
+// The split solve's scratch: the handle's and, after the factorisation, its working arrays.
+static Scratch solve_scratch(const BcrHandle* h) {
+  const int64_t bb = (int64_t)h->ny * h->ny * (int64_t)sizeof(double2), n1 = (h->nx + 1) / 2;
+  Scratch w;
+  w.add(h->scratch, std::max<int64_t>(h->m[0], 1) * bb);
+  for (void* a : {h->Dw[0], h->Dw[1], h->Lw[0], h->Lw[1]}) w.add(a, n1 * bb);
+  return w;
 }
 
 // One forward level in FP64: rows n of B (st elements apart), m eliminated.
-static cudaError_t split_fwd(BcrHandle* h, int cmax, const double2* Dinv, const double2* X, const double2* Y,
+static cudaError_t split_fwd(BcrHandle* h, Scratch& mem, const double2* Dinv, const double2* X, const double2* Y,
                              double2* B, int64_t st, double2* t, int n, int m, int nk, int nq, cudaStream_t s) {
   const int ny = h->ny, my = (n - 1) / 2;
   const int64_t nn = (int64_t)ny * ny, row = (int64_t)ny * nq;
-  const size_t f3 = sg_form_bytes(ny, ny, 3), fb = sg_form_bytes(nq, ny, 2);
-  const int ne = sg_form_exps(ny), nb = sg_form_exps(nq);
-  const int cb = (int)ceil_div(nk, ceil_div(nk, cmax));
+  const int cb = batch_of(mem, nk, [&](int c) { FwdBuf(mem, ny, nq, c); });
+  if (cb == 0) return cudaErrorInvalidValue;
   for (int k0 = 0; k0 < nk; k0 += cb) {
     const int c = std::min(cb, nk - k0), cm = std::min(c, m - k0), p0 = k0 > 0 ? 1 : 0;
     const int ny1 = std::max(0, std::min(k0 + c - 1, my) - (k0 - p0));  // Y of rows k0 - p0 .. k0 + c - 2
     const int nb1 = p0 + cm;                                            // odd rows from index k0 - p0 on
-    Carve w{(unsigned char*)h->scratch};
-    unsigned char* fD = w.take<unsigned char>(c * f3);
-    unsigned char* fX = w.take<unsigned char>(c * f3);
-    unsigned char* fY = w.take<unsigned char>((c + 1) * f3);
-    unsigned char* fB = w.take<unsigned char>((c + 1) * fb);
-    int32_t* eD = w.take<int32_t>(4 * (size_t)ne * c);
-    int32_t* eX = w.take<int32_t>(4 * (size_t)ne * c);
-    int32_t* eY = w.take<int32_t>(4 * (size_t)ne * (c + 1));
-    int32_t* eB = w.take<int32_t>(4 * (size_t)nb * (c + 1));
+    mem.reset();
+    const FwdBuf w(mem, ny, nq, c);
+    unsigned char *fD = w.D.f, *fX = w.X.f, *fY = w.Y.f, *fB = w.B.f;
+    int32_t *eD = w.D.e, *eX = w.X.e, *eY = w.Y.e, *eB = w.B.e;
     RCI_CUDA_TRY(launch_sg_split(Dinv + k0 * nn, false, ny, nn, false, ny, ny, 3, cm, fD, eD, nullptr, s));
     RCI_CUDA_TRY(launch_sg_split(X + k0 * nn, false, ny, nn, true, ny, ny, 3, cm, fX, eX, nullptr, s));
     RCI_CUDA_TRY(launch_sg_split(Y + (k0 - p0) * nn, false, ny, nn, true, ny, ny, 3, ny1, fY, eY, nullptr, s));
@@ -2583,22 +2656,19 @@ static cudaError_t split_fwd(BcrHandle* h, int cmax, const double2* Dinv, const 
 }
 
 // One backward level in FP64.
-static cudaError_t split_bwd(BcrHandle* h, int cmax, const double2* X, const double2* Y, double2* B, int64_t st,
+static cudaError_t split_bwd(BcrHandle* h, Scratch& mem, const double2* X, const double2* Y, double2* B, int64_t st,
                              const double2* t, int n, int m, int nq, cudaStream_t s) {
   const int ny = h->ny, my = (n - 1) / 2;
   const int64_t nn = (int64_t)ny * ny, row = (int64_t)ny * nq;
-  const size_t f3 = sg_form_bytes(ny, ny, 3), fb = sg_form_bytes(nq, ny, 2);
-  const int ne = sg_form_exps(ny), nb = sg_form_exps(nq), nk = (n + 1) / 2;
-  const int cb = (int)ceil_div(m, ceil_div(m, cmax));
+  const int nk = (n + 1) / 2;
+  const int cb = batch_of(mem, m, [&](int c) { FwdBuf(mem, ny, nq, c); });
+  if (cb == 0) return cudaErrorInvalidValue;
   for (int k0 = 0; k0 < m; k0 += cb) {
     const int c = std::min(cb, m - k0), cy = std::max(0, std::min(c, my - k0)), nb1 = std::min(c + 1, nk - k0);
-    Carve w{(unsigned char*)h->scratch};
-    unsigned char* fX = w.take<unsigned char>(c * f3);
-    unsigned char* fY = w.take<unsigned char>(c * f3);
-    unsigned char* fB = w.take<unsigned char>((c + 1) * fb);
-    int32_t* eX = w.take<int32_t>(4 * (size_t)ne * c);
-    int32_t* eY = w.take<int32_t>(4 * (size_t)ne * c);
-    int32_t* eB = w.take<int32_t>(4 * (size_t)nb * (c + 1));
+    mem.reset();
+    const FwdBuf w(mem, ny, nq, c);
+    unsigned char *fX = w.X.f, *fY = w.Y.f, *fB = w.B.f;
+    int32_t *eX = w.X.e, *eY = w.Y.e, *eB = w.B.e;
     RCI_CUDA_TRY(launch_sg_split(X + k0 * nn, false, ny, nn, false, ny, ny, 3, c, fX, eX, nullptr, s));
     RCI_CUDA_TRY(launch_sg_split(Y + k0 * nn, false, ny, nn, false, ny, ny, 3, cy, fY, eY, nullptr, s));
     RCI_CUDA_TRY(launch_sg_split(B + 2 * (int64_t)k0 * st, false, nq, 2 * st, true, nq, ny, 2, nb1, fB, eB, nullptr, s));
@@ -2647,8 +2717,13 @@ static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b
   sbytes += (double)nn * sizeof(cplx<T>) + 2.0 * nx * (double)ny * nrhs * sizeof(cplx<T>);
   const int dense = h->Lf - 1;
   ProfScope ps(h->prof, PF_SOLVE, s, sflops, sbytes, (m0 > 0 ? 1 : 0) + 1 + 2 * dense + 1 + dense + 1);
-  int cmax = 0;
-  if constexpr (sizeof(T) == 8) cmax = split_solve_batch(h, nq);
+  bool split = false;
+  Scratch mem;
+  if constexpr (sizeof(T) == 8) {
+    mem = solve_scratch(h);
+    FwdBuf(mem, ny, nq, 1);
+    split = ny <= SG_KMAX && !mem.full;
+  }
 
   // ---- level 0 forward by tridiagonal sweeps, then its kept rows
   if (m0 > 0) {
@@ -2669,8 +2744,8 @@ static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b
     const cplx<T>* Y = X + (int64_t)m * nn;
     const int64_t st = row << (l - 1);
     if constexpr (sizeof(T) == 8) {
-      if (cmax > 0) {
-        RCI_CUDA_TRY(split_fwd(h, cmax, Dinv, X, Y, B1, st, tl[l], n, m, nk, nq, s));
+      if (split) {
+        RCI_CUDA_TRY(split_fwd(h, mem, Dinv, X, Y, B1, st, tl[l], n, m, nk, nq, s));
         continue;
       }
     }
@@ -2684,12 +2759,11 @@ static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b
     const cplx<T>* Dinv = store + h->final_off;
     bool done = false;
     if constexpr (sizeof(T) == 8) {
-      if (cmax > 0) {
-        Carve w{(unsigned char*)h->scratch};
-        unsigned char* fD = w.take<unsigned char>(sg_form_bytes(ny, ny, 3));
-        unsigned char* fB = w.take<unsigned char>(sg_form_bytes(nq, ny, 2));
-        int32_t* eD = w.take<int32_t>(4 * (size_t)sg_form_exps(ny));
-        int32_t* eB = w.take<int32_t>(4 * (size_t)sg_form_exps(nq));
+      if (split) {
+        mem.reset();
+        const FwdBuf w(mem, ny, nq, 1);
+        unsigned char *fD = w.D.f, *fB = w.B.f;
+        int32_t *eD = w.D.e, *eB = w.B.e;
         RCI_CUDA_TRY(launch_sg_split(Dinv, false, ny, nn, false, ny, ny, 3, 1, fD, eD, nullptr, s));
         RCI_CUDA_TRY(launch_sg_split(B1, false, nq, row, true, nq, ny, 2, 1, fB, eB, nullptr, s));
         SgJob j{};
@@ -2716,8 +2790,8 @@ static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b
     const cplx<T>* Y = X + (int64_t)m * nn;
     const int64_t st = row << (l - 1);
     if constexpr (sizeof(T) == 8) {
-      if (cmax > 0) {
-        RCI_CUDA_TRY(split_bwd(h, cmax, X, Y, B1, st, tl[l], n, m, nq, s));
+      if (split) {
+        RCI_CUDA_TRY(split_bwd(h, mem, X, Y, B1, st, tl[l], n, m, nq, s));
         continue;
       }
     }
