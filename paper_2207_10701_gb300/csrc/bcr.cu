@@ -1031,7 +1031,7 @@ cudaError_t launch_gj_simt(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64
                            int n, int batch, int32_t* status, cudaStream_t s,
                            const int32_t* only = nullptr) {
   if (batch <= 0) return cudaSuccess;
-  if (n > 1024 || (only && (sizeof(T) == 4 || n > 256))) return cudaErrorInvalidValue;
+  if (n > 1024 || (only && ((sizeof(T) == 4 && n <= 160) || n > 256))) return cudaErrorInvalidValue;
   if constexpr (sizeof(T) == 4) {
     if (n <= 160 && GjLaSmem(n).total <= SMEM_LIMIT)
       return launch_gj_lookahead(src, src_stride, out, out_stride, n, batch, status, s);
@@ -1040,7 +1040,7 @@ cudaError_t launch_gj_simt(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64
                                                   status, s);
     if (n <= 256)
       return launch_gj_reg<T, false, 8, 5, 5, 512>(src, src_stride, out, out_stride, n, batch,
-                                                   status, s);
+                                                   status, s, only);
     return launch_gj_cfg<T, false, 16, 5, 5, 512>(src, src_stride, out, out_stride, n, batch,
                                                   status, s);
   } else {
@@ -2225,6 +2225,128 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
   return cudaSuccess;
 }
 
+// ---- FP32 blocks of more than 160 rows
+// A block of this size fits neither tensor memory nor shared memory, and the SIMT Gauss-Jordan kernel
+// works on it in L2 (7.8 us of the whole GPU a block of 224, 1.1 ms for one alone).  Instead:
+//   1. inversion by halves, A = [A11 A12; A21 A22]: P = A11^-1 and T = (A22 - A21 P A12)^-1 on the
+//      tensor-core Gauss-Jordan kernel, the products around them on the TMA-fed GEMM;
+//   2. pivoting only within the halves costs digits, so one Newton step X + X (I - A X) follows with
+//      the residual formed through the digit split (error 2^-36, where FP32 rounds at 2^-24): the
+//      inverse it leaves is closer to the exact one than the SIMT kernel's.
+// Blocks whose step would leave more than that kernel does (residual entries of some 1e-5 at n = 224),
+// or whose halves are singular, go to the SIMT kernel, which also reports zero pivots.
+namespace {
+
+// an h x h part of each of the blocks at src (rows lds apart) to dst (rows ldd apart)
+__global__ void block_part_kernel(const float2* __restrict__ src, int64_t ss, int lds, float2* __restrict__ dst,
+                                  int64_t sd, int ldd, int h, int64_t total) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= total) return;
+  const int64_t hh = (int64_t)h * h, z = e / hh, r = e - z * hh;
+  const int i = (int)(r / h), j = (int)(r - (int64_t)i * h);
+  dst[z * sd + (int64_t)i * ldd + j] = src[z * ss + (int64_t)i * lds + j];
+}
+
+// failed[z]: the residual R = I - A X of block z is too large for one Newton step
+__global__ void halves_check_kernel(const uint32_t* __restrict__ maxabs, int n, int batch, int32_t* failed,
+                                    const int32_t* __restrict__ st32, int32_t* status) {
+  const int z = blockIdx.x * blockDim.x + threadIdx.x;
+  if (z == 0 && *st32 == DEV_TIMEOUT) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+  if (z >= batch) return;
+  const float m = __uint_as_float(maxabs[z]);
+  failed[z] = (float)n * m * m <= 2e-6f ? 0 : 1;
+}
+
+struct HalvesBuf {
+  Form D, X;
+  float2 *X0, *P, *Q, *R, *S, *T, *res;  // res (n x n) takes the place of P .. T
+  int32_t* words;                        // maxabs, failed, status of the halves
+  int h1, h2;
+  HalvesBuf(Scratch& w, int n, size_t c) {
+    h1 = (int)ceil_div(n / 2, 16) * 16;
+    h2 = n - h1;
+    D = Form(w, n, n, 3, c);
+    X = Form(w, n, n, 2, c);
+    X0 = w.take<float2>(c * n * n * sizeof(float2));
+    const size_t a = c * h1 * h1, b = c * h1 * h2, d = c * h2 * h2;
+    P = w.take<float2>((2 * a + 2 * b + 2 * d) * sizeof(float2));  // 2 a: P and the packed A11
+    res = P;
+    Q = P + 2 * a;
+    R = Q + b;
+    S = R + b;
+    T = S + d;
+    words = w.take<int32_t>(4 * (2 * c + 1));
+  }
+};
+
+}  // namespace
+
+// out[z] = D[z]^-1 for z < m, FP32 blocks of 160 < ny <= SG_KMAX, even (D: stride elements apart,
+// destroyed where the SIMT kernel takes over).
+static cudaError_t halves_inverse(float2* D, int64_t stride, float2* out, int n, int m, Scratch& mem,
+                                  int32_t* status, cudaStream_t s) {
+  const int64_t nn = (int64_t)n * n;
+  const int cb = batch_of(mem, m, [&](int c) { HalvesBuf(mem, n, c); });
+  if (cb == 0) return cudaErrorInvalidValue;
+  const long long wl = tc_wait_limit();
+  // C[z] (M x N) = alpha A[z] B[z] (+ C0[z]), K terms
+  auto product = [&](int M, int N, int K, const float2* A, int64_t lda, int64_t sA, const float2* B, int64_t ldb,
+                     int64_t sB, float alpha, const float2* C0, int64_t ldc0, int64_t sC0, float2* C, int64_t ldc,
+                     int64_t sC, int c) {
+    return launch_tc_cgemm_tma(M, N, K, false, false, alpha, A, lda, sA, B, ldb, sB, C0 ? 1.f : 0.f, C0, ldc0, sC0, C,
+                               ldc, sC, c, status, wl, s);
+  };
+  for (int k0 = 0; k0 < m; k0 += cb) {
+    const int c = std::min(cb, m - k0);
+    mem.reset();
+    const HalvesBuf w(mem, n, c);
+    const int h1 = w.h1, h2 = w.h2;
+    const int64_t a = (int64_t)h1 * h1, b = (int64_t)h1 * h2, d = (int64_t)h2 * h2;
+    float2* A = D + (int64_t)k0 * stride;
+    float2 *A12 = A + h1, *A21 = A + (int64_t)h1 * n, *A22 = A21 + h1;
+    float2 *X0 = w.X0, *X12 = X0 + h1, *X21 = X0 + (int64_t)h1 * n, *X22 = X21 + h1;
+    float2 *P = w.P, *A11 = P + c * a;
+    uint32_t* maxabs = reinterpret_cast<uint32_t*>(w.words);
+    int32_t *failed = w.words + c, *st32 = w.words + 2 * c;
+    RCI_CUDA_TRY(cudaMemsetAsync(w.words, 0, sizeof(int32_t) * (2 * (size_t)c + 1), s));
+    block_part_kernel<<<(unsigned)ceil_div(c * a, 256), 256, 0, s>>>(A, stride, n, A11, a, h1, h1, c * a);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+    RCI_CUDA_TRY(launch_tc_gj(A11, a, P, a, h1, c, st32, s));
+    RCI_CUDA_TRY(product(h1, h2, h1, P, h1, a, A12, n, stride, 1.f, nullptr, 0, 0, w.Q, h2, b, c));
+    RCI_CUDA_TRY(product(h2, h1, h1, A21, n, stride, P, h1, a, 1.f, nullptr, 0, 0, w.R, h1, b, c));
+    RCI_CUDA_TRY(product(h2, h2, h1, A21, n, stride, w.Q, h2, b, -1.f, A22, n, stride, w.S, h2, d, c));
+    RCI_CUDA_TRY(launch_tc_gj(w.S, d, w.T, d, h2, c, st32, s));
+    RCI_CUDA_TRY(product(h1, h2, h2, w.Q, h2, b, w.T, h2, d, -1.f, nullptr, 0, 0, X12, n, nn, c));
+    RCI_CUDA_TRY(product(h2, h1, h2, w.T, h2, d, w.R, h1, b, -1.f, nullptr, 0, 0, X21, n, nn, c));
+    RCI_CUDA_TRY(product(h1, h1, h2, X12, n, nn, w.R, h1, b, -1.f, P, h1, a, X0, n, nn, c));
+    block_part_kernel<<<(unsigned)ceil_div(c * d, 256), 256, 0, s>>>(w.T, d, h2, X22, nn, n, h2, c * d);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+    // one Newton step
+    RCI_CUDA_TRY(launch_sg_split(A, true, n, stride, false, n, n, 3, c, w.D.f, w.D.e, nullptr, s, 5));
+    RCI_CUDA_TRY(launch_sg_split(X0, true, n, nn, true, n, n, 2, c, w.X.f, w.X.e, nullptr, s, 5));
+    SgJob r{};
+    r.nseg = 1;
+    r.seg[0] = SgSeg{w.D.f, w.D.e, w.X.f, w.X.e, 3, 2, 0, 0, 0, c};
+    r.neg = true;
+    r.identity = true;
+    r.C32 = w.res;
+    r.ldc = n;
+    r.sC = nn;
+    r.batch = c;
+    r.maxabs = maxabs;
+    RCI_CUDA_TRY(launch_sg_gemm(n, n, n, 1, &r, SG_HALF, status, wl, s));
+    halves_check_kernel<<<(unsigned)ceil_div(c, 128), 128, 0, s>>>(maxabs, n, c, failed, st32, status);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+    float2* X = out + (int64_t)k0 * nn;
+    RCI_CUDA_TRY(product(n, n, n, X0, n, nn, w.res, n, nn, 1.f, X0, n, nn, X, n, nn, c));
+    RCI_CUDA_TRY(launch_gj_simt<float>(A, stride, X, nn, n, c, status, s, failed));
+  }
+  return cudaSuccess;
+}
+
 // The products of one FP64 reduction level (the same five as the general path), in batches of
 // eliminated rows k0 .. k1 - 1:
 //   X_k = Dinv_k L_{2k+1};  Y_k = Dinv_k L_{2k+2}^T
@@ -2386,6 +2508,11 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
       split = batch_of(ws, 1, [&](int c) { LevelBuf(ws, ny, c); }) == 1;
     }
   }
+  // FP32 blocks above 160 rows by halves, where the scratch holds one
+  auto by_halves = [&](Scratch& w) {
+    return sizeof(T) == 4 && !h->simt && ny > 160 && ny <= SG_KMAX && ny % 2 == 0 &&
+           batch_of(w, 1, [&](int c) { HalvesBuf(w, ny, c); }) == 1;
+  };
   for (int l = 1; l < h->Lf; ++l) {
     const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
     const int my = (n - 1) / 2;
@@ -2406,7 +2533,17 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
           RCI_CUDA_TRY(split_inverse(D + nn, 2 * nn, Dinv, ny, m, w, h->status, s));
         }
       }
-      if (!split) RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
+      bool halves = false;
+      if constexpr (sizeof(T) == 4) {
+        Scratch w = scratch_of(l, false);
+        if (by_halves(w)) {
+          RCI_CUDA_TRY(launch_block_maxabs<T>(D + nn, 2 * nn, nn, m, maxabs + 1, s));
+          const cudaError_t e = halves_inverse(D + nn, 2 * nn, Dinv, ny, m, w, h->status, s);
+          if (e != cudaSuccess && e != cudaErrorNotSupported) return e;
+          halves = e == cudaSuccess;
+        }
+      }
+      if (!split && !halves) RCI_CUDA_TRY(launch_gj<T>(D + nn, 2 * nn, Dinv, nn, ny, m, h->status, s, maxabs + 1,
                                 !h->simt));
     }
     // X_k = Dinv_k L_{2k+1};  Y_k = Dinv_k L_{2k+2}^T
@@ -2497,6 +2634,14 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
         RCI_CUDA_TRY(launch_block_maxabs<T>((cplx<T>*)h->Dw[cur], nn, nn, 1, maxabs + 1, s));
         Scratch w = scratch_of(h->Lf, false);
         return split_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, w, h->status, s);
+      }
+    }
+    if constexpr (sizeof(T) == 4) {
+      Scratch w = scratch_of(h->Lf, false);
+      if (by_halves(w)) {
+        RCI_CUDA_TRY(launch_block_maxabs<T>((cplx<T>*)h->Dw[cur], nn, nn, 1, maxabs + 1, s));
+        const cudaError_t e = halves_inverse((cplx<T>*)h->Dw[cur], nn, store + h->final_off, ny, 1, w, h->status, s);
+        if (e != cudaErrorNotSupported) return e;
       }
     }
     RCI_CUDA_TRY(launch_gj<T>((cplx<T>*)h->Dw[cur], 0, store + h->final_off, 0, ny, 1, h->status, s,

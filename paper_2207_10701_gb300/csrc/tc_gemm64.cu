@@ -444,7 +444,6 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
         const double2* C0 = first ? (jb.C0 ? jb.C0 + tl.z * jb.sC0 : nullptr) : jb.C + tl.z * jb.sC;
         const int64_t ldc0 = first ? jb.ldc0 : jb.ldc;
         const bool eye = first && jb.identity;
-        const bool add = eye || C0 != nullptr;
         // the columns' exponents (the threads that read the last pass's are past a barrier since)
         if (et < p.nt) sh_eb[et] = tl.n0 + et < p.N ? eB[tl.n0 + et] : 0;
         double2* C = jb.C + tl.z * jb.sC;
@@ -495,7 +494,6 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
           for (int i = 0; i < 2; ++i) {
             const int gr = tl.i0 + r + 32 * i;
             c0[i] = (C0 && gr < p.M && col < p.N) ? C0[(int64_t)gr * ldc0 + col] : make_double2(0.0, 0.0);
-            if (eye && gr == col) c0[i].x = 1.0;
           }
           double* sp = reinterpret_cast<double*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES) +
                        (row * SG_STG_LD + c4) * 2 + part;
@@ -513,11 +511,14 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
                 o.x = -o.x;
                 o.y = -o.y;
               }
-              if (add) {
+              if (eye) {
+                if (gr == col) o.x += 1.0;
+              } else if (C0) {
                 o.x += c0[i].x;
                 o.y += c0[i].y;
               }
-              C[(int64_t)gr * jb.ldc + col] = o;
+              if (jb.C32) jb.C32[tl.z * jb.sC + (int64_t)gr * jb.ldc + col] = make_float2((float)o.x, (float)o.y);
+              else C[(int64_t)gr * jb.ldc + col] = o;
               big = max(big, max((uint32_t)__double2hiint(o.x) & 0x7fffffffu,
                                  (uint32_t)__double2hiint(o.y) & 0x7fffffffu));
             }
@@ -573,7 +574,7 @@ template <typename T>
 __global__ void __launch_bounds__(SS_THREADS)
 sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int trans, int rows, int K,
                 int planes, int chunks, int G, unsigned char* __restrict__ form, int32_t* __restrict__ exps,
-                const int32_t* __restrict__ skip) {
+                const int32_t* __restrict__ skip, int digits) {
   extern __shared__ __align__(16) unsigned char raw[];
   const int z = blockIdx.y;
   if (skip && skip[z]) return;
@@ -632,6 +633,7 @@ sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int
     float w = 1.f;
 #pragma unroll
     for (int s = 0; s < SG_SLICES; ++s) {
+      if (s >= digits) break;
       float d[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
@@ -684,7 +686,7 @@ size_t sg_form_bytes(int rows, int K, int planes) {
 
 cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t stride, bool trans,
                             int rows, int K, int planes, int batch, unsigned char* form,
-                            int32_t* exps, const int32_t* skip, cudaStream_t s) {
+                            int32_t* exps, const int32_t* skip, cudaStream_t s, int digits) {
   if (batch <= 0) return cudaSuccess;
   if (rows < 1 || K < 1 || K > SG_KMAX || batch > 65535 || (planes != 2 && planes != 3))
     return cudaErrorInvalidValue;
@@ -693,13 +695,13 @@ cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t strid
   const dim3 grid((unsigned)ceil_div(rows, SS_ROWS), (unsigned)batch);
   if (f32) {
     sg_split_kernel<float><<<grid, SS_THREADS, smem, s>>>((const float2*)src, ld, stride, trans ? 1 : 0, rows, K,
-                                                          planes, chunks, G, form, exps, skip);
+                                                          planes, chunks, G, form, exps, skip, digits);
   } else {
     if (smem > 48 * 1024)
       RCI_CUDA_TRY(cudaFuncSetAttribute(sg_split_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)smem));
     sg_split_kernel<double><<<grid, SS_THREADS, smem, s>>>((const double2*)src, ld, stride, trans ? 1 : 0, rows, K,
-                                                           planes, chunks, G, form, exps, skip);
+                                                           planes, chunks, G, form, exps, skip, digits);
   }
   rci_note_launch();
   return cudaGetLastError();
@@ -745,7 +747,7 @@ cudaError_t launch_sg_gemm(int M, int N, int K, int njob, const SgJob* jobs, SgD
   for (int j = 0; j < njob; ++j) {
     const SgJob& q = jobs[j];
     if (q.batch <= 0) continue;
-    if (q.nseg < 1 || q.nseg > 2) return cudaErrorInvalidValue;
+    if (q.nseg < 1 || q.nseg > 2 || (q.C32 && (q.nseg > 1 || q.C0))) return cudaErrorInvalidValue;
     for (int g = 0; g < q.nseg; ++g)
       if (q.seg[g].planesA != 3 || q.seg[g].planesB < 2) return cudaErrorInvalidValue;
     a.job[a.njob++] = q;

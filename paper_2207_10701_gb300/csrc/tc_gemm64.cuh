@@ -17,9 +17,10 @@ inline int sg_form_exps(int rows) { return (int)ceil_div(rows, 8) * 8; }
 // Split `batch` operands: row r, term k of operand z is src[z][r][k] (trans == false) or
 // src[z][k][r] (trans), row-major with leading dimension ld and `stride` complex elements between
 // the operands; src is complex64 (f32) or complex128.  Operands whose skip[z] != 0 are left out.
+// digits: the highest of the seven digits that are written (five serve SG_HALF).
 cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t stride, bool trans,
                             int rows, int K, int planes, int batch, unsigned char* form,
-                            int32_t* exps, const int32_t* skip, cudaStream_t s);
+                            int32_t* exps, const int32_t* skip, cudaStream_t s, int digits = SG_SLICES);
 
 // One term of a product set: output z (zlo <= z < zhi) adds A[z + zA] B[z + zB]^T of the split
 // forms (members contiguous).
@@ -34,7 +35,8 @@ struct SgSeg {
 
 // C[z] = C0[z] +- sum_g A_g B_g^T  (M x N outputs, K terms; neg: minus; C0 null: nothing added;
 // C may be C0).  Every output takes part in at least one segment.  identity: C0 is the identity
-// matrix.  maxabs[z] (or null): atomicMax of the bits of the largest |re|, |im| of output z as a
+// matrix.  C32 in the place of C: outputs rounded to complex64 (one segment, C0 null).
+// maxabs[z] (or null): atomicMax of the bits of the largest |re|, |im| of output z as a
 // float (rounded up by less than 2^-20; infinity for anything not finite).
 // Products with skip[z] != 0 (or null) are left out, C[z] untouched; *any == 0 (or null) says that
 // all of a one-job launch are.
@@ -45,6 +47,7 @@ struct SgJob {
   const double2* C0;
   int64_t ldc0, sC0;
   double2* C;
+  float2* C32;
   int64_t ldc, sC;
   int batch;
   uint32_t* maxabs;
