@@ -18,6 +18,26 @@ __host__ __device__ size_t tri_smem_per_warp(int ny) {
   return ((size_t)6 * ny * sizeof(cplx<T>) + (size_t)ny + 15) & ~(size_t)15;
 }
 
+// 1 / a by one division: scaled by a power of two (exactly) so that |a|^2 neither overflows nor
+// underflows.  The general crecip divides four times, one after the other; in the serial
+// elimination below that was most of a step.
+__device__ __forceinline__ double pow2_of(double a, double b, int sign) {
+  const int e = max((__double2hiint(a) >> 20) & 0x7ff, (__double2hiint(b) >> 20) & 0x7ff) - 1023;
+  return __hiloint2double((1023 + sign * max(-1000, min(1000, e))) << 20, 0);
+}
+__device__ __forceinline__ float pow2_of(float a, float b, int sign) {
+  const int e = max((__float_as_int(a) >> 23) & 0xff, (__float_as_int(b) >> 23) & 0xff) - 127;
+  return __int_as_float((127 + sign * max(-120, min(120, e))) << 23);
+}
+template <typename C>
+__device__ __forceinline__ C crecip1(C a) {
+  const auto f = pow2_of(a.x, a.y, -1);
+  const auto ar = a.x * f, ai = a.y * f;
+  const auto r = (decltype(f))1 / (ar * ar + ai * ai);
+  if (ar == 0 && ai == 0) return a - a;  // 0 / 0: zero, as crecip
+  return mkc((ar * r) * f, -(ai * r) * f);
+}
+
 // Pivoted LU of the tridiagonal diagonal block T_r of an eliminated row r = 2k+1
 // (Gaussian elimination with adjacent-row interchanges): multipliers dl, inverse
 // pivots dinv, first and second superdiagonals du, du2 of U, and swap flags piv.
@@ -56,7 +76,7 @@ tri_factor_kernel(const double2* __restrict__ dg, const double2* __restrict__ cy
       const cplx<T> dunext = (j + 1 < ny - 1) ? o[j + 1] : czero<T>();
       if (cabs1(cur_d) >= cabs1(bs)) {
         if (cabs1(cur_d) == T(0)) sing = true;
-        const cplx<T> inv = crecip(cur_d);
+        const cplx<T> inv = crecip1(cur_d);
         const cplx<T> m = bs * inv;
         dl[j] = m;
         di[j] = inv;
@@ -66,7 +86,7 @@ tri_factor_kernel(const double2* __restrict__ dg, const double2* __restrict__ cy
         cur_d = dnext - m * cur_du;
         cur_du = dunext;
       } else {
-        const cplx<T> inv = crecip(bs);
+        const cplx<T> inv = crecip1(bs);
         const cplx<T> m = cur_d * inv;
         dl[j] = m;
         di[j] = inv;
@@ -78,7 +98,7 @@ tri_factor_kernel(const double2* __restrict__ dg, const double2* __restrict__ cy
       }
     }
     if (cabs1(cur_d) == T(0)) sing = true;
-    di[ny - 1] = crecip(cur_d);
+    di[ny - 1] = crecip1(cur_d);
     dl[ny - 1] = czero<T>();
     du[ny - 1] = czero<T>();
     du2[ny - 1] = czero<T>();
@@ -167,8 +187,12 @@ __device__ __forceinline__ void tri_forward_unit(const TriRow<T>& f, int n, int 
 // two scratch columns (YR, YL: the next level's free working arrays; only the rows from
 // b - 1 on, the others being zero), then one backward sweep runs both recurrences side by
 // side, so that every entry of D'_k is formed in one step (no read-back of a partial D'),
-// with the scratch loads issued a few rows ahead.
-template <typename T>
+// with the scratch loads issued a few rows ahead.  D' and L' are symmetric (the couplings are
+// products of a factor of the row and one of the column).  HALF: a thread stops at the diagonal
+// and mirror_kernel fills the upper triangles.  That pays where the FP64 pipe bounds the kernel
+// (2020 rows of 160: 4.70 -> 3.12 + 0.28 ms), not in FP32 (0.52 -> 0.47 + 0.19), whose threads wait
+// for the longest one anyway.
+template <typename T, bool HALF>
 __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double2* __restrict__ cx,
                                     const double2* __restrict__ cy, int nx, int ny,
                                     const cplx<T>* __restrict__ tdl, const cplx<T>* __restrict__ tdinv,
@@ -242,11 +266,12 @@ __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double
     yr[q] = (has_r && a >= a_lo) ? YR[(int64_t)a * ny] : czero<T>();
     yl[q] = (has_l && a >= a_lo) ? YL[(int64_t)a * ny] : czero<T>();
   }
-  for (int a0 = ny - 1; a0 >= 0; a0 -= PF) {
+  const int a_end = HALF ? b : 0;
+  for (int a0 = ny - 1; a0 >= a_end; a0 -= PF) {
 #pragma unroll
     for (int q = 0; q < PF; ++q) {
       const int a = a0 - q;
-      if (a < 0) break;
+      if (a < a_end) break;
       const cplx<T> cr = yr[q], cl = yl[q];
       const int an = a - PF;  // the row PF steps ahead into the same ring slot
       yr[q] = (has_r && an >= a_lo) ? YR[(int64_t)an * ny] : czero<T>();
@@ -265,6 +290,29 @@ __global__ void level0_schur_kernel(const double2* __restrict__ dg, const double
       Dcol[(int64_t)a * ny] = cfms(cgl, sl, cfms(cxr[a] * gr, sb, te));
       if (has_l) Lcol[(int64_t)a * ny] = -(cgl * sl2);
     }
+  }
+}
+
+// M[z][b][a] = M[z][a][b] for a > b: the upper triangles of the n x n blocks of two arrays from their
+// lower ones, a 32 x 32 tile per block through shared memory.
+template <typename T>
+__global__ void __launch_bounds__(256)
+mirror_kernel(cplx<T>* __restrict__ D, cplx<T>* __restrict__ L, int n, int first_l) {
+  __shared__ cplx<T> t[32][33];
+  const int z = blockIdx.y;
+  if (blockIdx.z == 1 && z < first_l) return;
+  cplx<T>* M = (blockIdx.z == 0 ? D : L) + (int64_t)z * n * n;
+  int ta = 0, tb = blockIdx.x;  // tile row ta >= tile column tb
+  while (tb > ta) tb -= ++ta;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int i = ty; i < 32; i += 8) {
+    const int a = 32 * ta + i, b = 32 * tb + tx;
+    if (a < n && b < n) t[i][tx] = M[(int64_t)a * n + b];
+  }
+  __syncthreads();
+  for (int i = ty; i < 32; i += 8) {
+    const int b = 32 * tb + i, a = 32 * ta + tx;
+    if (a < n && a > b) M[(int64_t)b * n + a] = t[tx][i];
   }
 }
 
@@ -2466,17 +2514,26 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
   }
   {
     // D' and L' of the first reduced system
+    constexpr bool half = sizeof(T) == 8;
     const int thr = (int)ceil_div(ny, 32) * 32;
     const size_t smem = l0_smem<T>(ny);
     if (smem > 48 * 1024)
-      RCI_CUDA_TRY(cudaFuncSetAttribute(level0_schur_kernel<T>,
+      RCI_CUDA_TRY(cudaFuncSetAttribute(level0_schur_kernel<T, half>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // the next level's working arrays are free during level 0 and serve as scratch
-    level0_schur_kernel<T><<<n1, thr, smem, s>>>(dg, cx, cy, nx, ny, tdl, tdinv, tdu, tdu2,
+    level0_schur_kernel<T, half><<<n1, thr, smem, s>>>(dg, cx, cy, nx, ny, tdl, tdinv, tdu, tdu2,
                                                     h->tpiv, (cplx<T>*)h->Dw[0], (cplx<T>*)h->Lw[0],
                                                     (cplx<T>*)h->Dw[1], (cplx<T>*)h->Lw[1]);
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
+    const int tiles = (int)ceil_div(ny, 32);
+    for (int z0 = 0; half && z0 < n1; z0 += 32768) {  // (a grid's second extent ends at 65535)
+      const int nz = std::min(n1 - z0, 32768);
+      mirror_kernel<T><<<dim3((unsigned)(tiles * (tiles + 1) / 2), (unsigned)nz, 2), 256, 0, s>>>(
+          (cplx<T>*)h->Dw[0] + z0 * nn, (cplx<T>*)h->Lw[0] + z0 * nn, ny, z0 == 0 ? 1 : 0);
+      rci_note_launch();
+      RCI_CUDA_TRY(cudaGetLastError());
+    }
   }
   delete l0;
   const cplx<T> one = mkc(T(1), T(0)), mone = mkc(T(-1), T(0)), zero = czero<T>();
@@ -3029,12 +3086,22 @@ static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, 
                                                          (int)trs_smem)
                                   : cudaSuccess;
     };
+    // Many FP64 rows: one thread per row.  The FP64 pipe takes as long for a warp's one busy lane as for
+    // all of them, so with a warp per row 2020 rows of 160 take 340 us a sweep; with a thread per row
+    // 235 and 255.  Few rows are bound by one row's chain of operations, which is shorter on a warp's
+    // staged copies (220 rows of 128: 84 us against 170 and 200).
+    const bool thread_per_row = sizeof(T) == 8 && m0 > 1024;
     if (m0 > 0) {
-      RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, false>));
-      tri_rows_solve_kernel<T, false><<<(unsigned)ceil_div(m0, TRS_WARPS), 32 * TRS_WARPS,
-                                        trs_smem, s>>>(
-          (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
-          (const cplx<T>*)h->tdu2, h->tpiv, bsrc, nullptr, cx, t0, nx, ny, m0);
+      if (thread_per_row) {
+        fwd0_kernel<T><<<(unsigned)ceil_div(m0, 32), 32, 0, s>>>(
+            bsrc, t0, ny, m0, 1, 1, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+            (const cplx<T>*)h->tdu2, h->tpiv);
+      } else {
+        RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, false>));
+        tri_rows_solve_kernel<T, false><<<(unsigned)ceil_div(m0, TRS_WARPS), 32 * TRS_WARPS, trs_smem, s>>>(
+            (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+            (const cplx<T>*)h->tdu2, h->tpiv, bsrc, nullptr, cx, t0, nx, ny, m0);
+      }
       rci_note_launch();
       RCI_CUDA_TRY(cudaGetLastError());
     }
@@ -3084,11 +3151,16 @@ static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, 
                         B[l + 1], B[l], n, m, ny);
     }
     // ---- level 0 backward by tridiagonal sweeps (and the kept rows copied)
-    RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, true>));
-    tri_rows_solve_kernel<T, true><<<(unsigned)ceil_div(n1, TRS_WARPS), 32 * TRS_WARPS,
-                                     trs_smem, s>>>(
-        (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
-        (const cplx<T>*)h->tdu2, h->tpiv, bsrc, B[1], cx, x, nx, ny, n1);
+    if (thread_per_row) {
+      bwd0_kernel<T><<<(unsigned)ceil_div(n1, 32), 32, 0, s>>>(
+          bsrc, B[1], cx, x, nx, ny, n1, 1, 1, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv,
+          (const cplx<T>*)h->tdu, (const cplx<T>*)h->tdu2, h->tpiv);
+    } else {
+      RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, true>));
+      tri_rows_solve_kernel<T, true><<<(unsigned)ceil_div(n1, TRS_WARPS), 32 * TRS_WARPS, trs_smem, s>>>(
+          (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+          (const cplx<T>*)h->tdu2, h->tpiv, bsrc, B[1], cx, x, nx, ny, n1);
+    }
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
 #undef RCI_SMAX_DISPATCH

@@ -187,11 +187,12 @@ __global__ void vf_tables_kernel(GridGeom g, int D, const double* __restrict__ g
 // anchor serves 64 columns, a block VF_GROUP anchors and a chunk of the nodes: per node it
 // evaluates 2 sincos for each anchor and 2 for each of the 32 distances instead of 2 cosines for
 // each column, and 3 FMAs per node and column remain.  The rounding of k (x_f - x_c) is that of
-// the direct form's argument.  Bound by the FP64 pipe: 2.67 -> 0.4 ms at 4000 columns (one cosine
+// the direct form's argument.  Bound by the FP64 pipe: 2.67 -> 0.28 ms at 4000 columns (one cosine
 // per node and column: 65.5 million of them).  The chunks' sums are added in a fixed order.
 constexpr int VF_SIDE = 32;            // columns on either side of an anchor
 constexpr int VF_WARPS = 8, VF_PER_WARP = 4, VF_GROUP = VF_WARPS * VF_PER_WARP;
 constexpr int VF_TILE = 16;            // nodes staged at a time
+constexpr double VF_NONE = 1e-33;
 
 __global__ void __launch_bounds__(32 * VF_WARPS)
 vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes,
@@ -202,14 +203,18 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
   const int a0 = blockIdx.x * VF_GROUP;
   double er[VF_PER_WARP] = {}, ei[VF_PER_WARP] = {}, orr[VF_PER_WARP] = {}, oi[VF_PER_WARP] = {};
   for (int n0 = blockIdx.y * nodes; n0 < (int)(blockIdx.y + 1) * nodes; n0 += VF_TILE) {
-    __syncthreads();
+    // evanescent nodes that have decayed below VF_NONE on the way count for nothing beside the
+    // propagating ones (weights of some 1e-3): 60 % of them at 100 rows, 85 % at 400
+    const bool ev = __syncthreads_or(threadIdx.x < VF_TILE &&
+                                     fabs(tab[4 * VF_NODES + 2 * (n0 + threadIdx.x) + 1]) >= VF_NONE);
     for (int e = threadIdx.x; e < VF_TILE * VF_SIDE; e += 32 * VF_WARPS) {
       const int n = n0 + e / VF_SIDE, j = e % VF_SIDE;
       const double d = ((double)j + 0.5) * g.h;
       double2 u, v;
       sincos(tab[4 * n] * d, &u.y, &u.x);
-      sincos(tab[4 * VF_NODES + 2 * n] * d, &v.y, &v.x);
       qp[e / VF_SIDE][j] = u;
+      if (!ev) continue;
+      sincos(tab[4 * VF_NODES + 2 * n] * d, &v.y, &v.x);
       qe[e / VF_SIDE][j] = v;
     }
     for (int e = threadIdx.x; e < VF_GROUP * VF_TILE; e += 32 * VF_WARPS) {
@@ -223,6 +228,7 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
       o[1] = fi * c;
       o[2] = fr * s;
       o[3] = fi * s;
+      if (!ev) continue;
       sincos(tab[4 * VF_NODES + 2 * n] * delta, &s, &c);
       const double fe = tab[4 * VF_NODES + 2 * n + 1];
       o[4] = fe * c;
@@ -231,7 +237,7 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
     __syncthreads();
 #pragma unroll 2
     for (int n = 0; n < VF_TILE; ++n) {
-      const double2 u = qp[n][lane], v = qe[n][lane];
+      const double2 u = qp[n][lane];
 #pragma unroll
       for (int i = 0; i < VF_PER_WARP; ++i) {
         const double* o = pc[warp * VF_PER_WARP + i][n];
@@ -239,6 +245,15 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
         ei[i] = fma(o[1], u.x, ei[i]);
         orr[i] = fma(o[2], u.y, orr[i]);
         oi[i] = fma(o[3], u.y, oi[i]);
+      }
+    }
+    if (!ev) continue;
+#pragma unroll 2
+    for (int n = 0; n < VF_TILE; ++n) {
+      const double2 v = qe[n][lane];
+#pragma unroll
+      for (int i = 0; i < VF_PER_WARP; ++i) {
+        const double* o = pc[warp * VF_PER_WARP + i][n];
         er[i] = fma(o[4], v.x, er[i]);
         orr[i] = fma(o[5], v.y, orr[i]);
       }
@@ -258,6 +273,7 @@ __global__ void vf_join_kernel(GridGeom g, const double2* __restrict__ part, int
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= g.n_src) return;
   double ar = 0.0, ai = 0.0;
+#pragma unroll 16
   for (int c = 0; c < chunks; ++c) {
     const double2 v = part[(int64_t)c * g.n_src + t];
     ar += v.x;
@@ -406,8 +422,8 @@ cudaError_t launch_virtual_focus_row(const GridGeom& g, double x_f, int d_rows, 
   if (!have_rule) RCI_CUDA_TRY(launch_gauss_legendre(VF_ORDER, -1.0, 1.0, gx, gw, s));
   vf_tables_kernel<<<(unsigned)ceil_div(VF_NODES, 128), 128, 0, s>>>(g, d_rows, gx, gw, tab); rci_note_launch();
   RCI_CUDA_TRY(cudaGetLastError());
-  // 64 chunks of 128 nodes where the scratch holds as many partial rows (ny >= 64), else fewer
-  int chunks = 64;
+  // 128 chunks of 64 nodes where the scratch holds as many partial rows (ny >= 128), else fewer
+  int chunks = 128;
   while (chunks > g.ny) chunks >>= 1;
   const unsigned groups = (unsigned)ceil_div(g.n_src, 2 * VF_SIDE * VF_GROUP);
   vf_sums_kernel<<<dim3(groups, (unsigned)chunks), 32 * VF_WARPS, 0, s>>>(g, x_f, tab, VF_NODES / chunks, part);

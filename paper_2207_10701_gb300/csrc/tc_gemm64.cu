@@ -548,13 +548,13 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
 }
 
 // ---------------------------------------------------------------- split
-// One block: 16 rows (two groups) of one operand.  The rows are staged in shared memory with
-// coalesced reads in either orientation, the row exponents reduced over 16 threads each, then a
+// One block: ROWS rows (one or two groups) of one operand.  The rows are staged in shared memory with
+// coalesced reads in either orientation, the row exponents reduced over 256 / ROWS threads each, then a
 // thread takes eight consecutive terms of a row: the value as a 56-bit fixed-point integer, its
 // balanced base-256 digits as the bytes of q + 0x808080808080, turned into floats by a byte
 // permute and one FMA each, and stored as 16-byte core-matrix rows (16 threads cover 256
 // contiguous bytes).  Bound by the integer issue rate: about 30 instructions per real.
-constexpr int SS_ROWS = 16, SS_THREADS = 256;
+constexpr int SS_THREADS = 256;
 
 __device__ __forceinline__ long long fixed56(double x, int e) {
   // x = m 2^(p - 52), |x| < 2^e; q = rint(x 2^(55 - e))
@@ -570,7 +570,7 @@ __device__ __forceinline__ long long fixed56(double x, int e) {
   return b < 0 ? -q : q;
 }
 
-template <typename T>
+template <typename T, int SS_ROWS>
 __global__ void __launch_bounds__(SS_THREADS)
 sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int trans, int rows, int K,
                 int planes, int chunks, int G, unsigned char* __restrict__ form, int32_t* __restrict__ exps,
@@ -596,15 +596,16 @@ sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int
   }
   __syncthreads();
   {
-    const int r = threadIdx.x >> 4, l = threadIdx.x & 15;
+    constexpr int W = SS_THREADS / SS_ROWS;  // 16 or 32 threads a row
+    const int r = threadIdx.x / W, l = threadIdx.x % W;
     int m = 0;
-    for (int k = l; k < Kp; k += 16) {
+    for (int k = l; k < Kp; k += W) {
       const cplx<T> v = t[r * LD + k];
       const int a = (__double2hiint((double)v.x) >> 20) & 0x7ff, b = (__double2hiint((double)v.y) >> 20) & 0x7ff;
       m = max(m, max(a, b));
     }
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int o = W / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     // biased exponent p of the largest entry: every |x| < 2^(p - 1022)
     if (l == 0) {
       const int e = m == 0x7ff ? SG_EXP_NONFINITE : (m == 0 ? 0 : m - 1022);
@@ -618,8 +619,10 @@ sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int
   unsigned char* F = form + (int64_t)z * fbytes;
   const int g0 = r0 >> 3;
   // item: row-in-group (8) | term half (2) | group (2) | part (2) | chunk
-  for (int it = threadIdx.x; it < chunks * 64; it += SS_THREADS) {
-    const int rr = it & 7, kc = (it >> 3) & 1, gg = (it >> 4) & 1, part = (it >> 5) & 1, c = it >> 6;
+  for (int it = threadIdx.x; it < chunks * 4 * SS_ROWS; it += SS_THREADS) {
+    constexpr int GL = SS_ROWS == 16 ? 1 : 0;  // bits of the group
+    const int rr = it & 7, kc = (it >> 3) & 1, gg = GL ? (it >> 4) & 1 : 0, part = (it >> (4 + GL)) & 1,
+              c = it >> (5 + GL);
     const int r = gg * 8 + rr;
     if (g0 + gg >= G) continue;
     const int e = re[r];
@@ -691,20 +694,22 @@ cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t strid
   if (rows < 1 || K < 1 || K > SG_KMAX || batch > 65535 || (planes != 2 && planes != 3))
     return cudaErrorInvalidValue;
   const int chunks = (int)ceil_div(K, 16), G = (int)ceil_div(rows, 8);
-  const size_t smem = (size_t)SS_ROWS * (chunks * 16 + 1) * (f32 ? sizeof(float2) : sizeof(double2));
-  const dim3 grid((unsigned)ceil_div(rows, SS_ROWS), (unsigned)batch);
-  if (f32) {
-    sg_split_kernel<float><<<grid, SS_THREADS, smem, s>>>((const float2*)src, ld, stride, trans ? 1 : 0, rows, K,
-                                                          planes, chunks, G, form, exps, skip, digits);
-  } else {
+  // 16 rows a block; 8 where those blocks do not go twice round the SMs (a batch of one operand of
+  // 128 rows: 6 -> 4 us)
+  const bool few = (int64_t)ceil_div(rows, 16) * batch < 2 * sm_count();
+  const int per = few ? 8 : 16;
+  const size_t smem = (size_t)per * (chunks * 16 + 1) * (f32 ? sizeof(float2) : sizeof(double2));
+  const dim3 grid((unsigned)ceil_div(rows, per), (unsigned)batch);
+  auto go = [&](auto kernel, auto* p) -> cudaError_t {
     if (smem > 48 * 1024)
-      RCI_CUDA_TRY(cudaFuncSetAttribute(sg_split_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem));
-    sg_split_kernel<double><<<grid, SS_THREADS, smem, s>>>((const double2*)src, ld, stride, trans ? 1 : 0, rows, K,
-                                                           planes, chunks, G, form, exps, skip, digits);
-  }
-  rci_note_launch();
-  return cudaGetLastError();
+      RCI_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<grid, SS_THREADS, smem, s>>>(p, ld, stride, trans ? 1 : 0, rows, K, planes, chunks, G, form, exps, skip,
+                                          digits);
+    rci_note_launch();
+    return cudaGetLastError();
+  };
+  if (f32) return few ? go(sg_split_kernel<float, 8>, (const float2*)src) : go(sg_split_kernel<float, 16>, (const float2*)src);
+  return few ? go(sg_split_kernel<double, 8>, (const double2*)src) : go(sg_split_kernel<double, 16>, (const double2*)src);
 }
 
 namespace {
