@@ -2234,7 +2234,7 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
     for (int it = 0; it < NEWTON_STEPS; ++it) {
       const NewtonFlags fl{reinterpret_cast<uint32_t*>(words), words + c, words + 2 * c, words + 3 * c,
                            st32 + 1 + 2 * it};
-      RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, true, ny, ny, 2, c, fXc, eXc, fl.skip_r, s));
+      RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, true, ny, ny, 2, c, fXc, eXc, fl.skip_r, s, it == 0 ? 5 : SG_SLICES));
       SgJob r{};
       r.nseg = 1;
       r.seg[0] = SgSeg{fD, eD, fXc, eXc, 3, 2, 0, 0, 0, c};
@@ -2252,8 +2252,11 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
                                                                      st32, status);
       rci_note_launch();
       RCI_CUDA_TRY(cudaGetLastError());
-      RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, false, ny, ny, 3, c, fXr, eXr, fl.skip_x, s));
-      RCI_CUDA_TRY(launch_sg_split(R, false, ny, nn, true, ny, ny, 2, c, fR, eR, fl.skip_x, s));
+      // (the first update corrects some 1e-5 and takes SG_HALF; the later ones correct 1e-8 or less)
+      const SgDigits du = it == 0 ? SG_HALF : SG_SMALL;
+      const int nd = it == 0 ? 5 : 4;
+      RCI_CUDA_TRY(launch_sg_split(X, false, ny, nn, false, ny, ny, 3, c, fXr, eXr, fl.skip_x, s, nd));
+      RCI_CUDA_TRY(launch_sg_split(R, false, ny, nn, true, ny, ny, 2, c, fR, eR, fl.skip_x, s, nd));
       SgJob x{};
       x.nseg = 1;
       x.seg[0] = SgSeg{fXr, eXr, fR, eR, 3, 2, 0, 0, 0, c};
@@ -2266,7 +2269,7 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
       x.batch = c;
       x.skip = fl.skip_x;
       x.any = &fl.active[0];
-      RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &x, SG_HALF, status, wl, s));
+      RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &x, du, status, wl, s));
     }
     RCI_CUDA_TRY(launch_gj_simt<double>(Dk, stride, X, nn, ny, c, status, s, words + 3 * c));
   }
@@ -2279,7 +2282,7 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
 //   1. inversion by halves, A = [A11 A12; A21 A22]: P = A11^-1 and T = (A22 - A21 P A12)^-1 on the
 //      tensor-core Gauss-Jordan kernel, the products around them on the TMA-fed GEMM;
 //   2. pivoting only within the halves costs digits, so one Newton step X + X (I - A X) follows with
-//      the residual formed through the digit split (error 2^-36, where FP32 rounds at 2^-24): the
+//      the residual formed through the digit split (SG_SMALL: error 2^-28, where FP32 rounds at 2^-24): the
 //      inverse it leaves is closer to the exact one than the SIMT kernel's.
 // Blocks whose step would leave more than that kernel does (residual entries of some 1e-5 at n = 224),
 // or whose halves are singular, go to the SIMT kernel, which also reports zero pivots.
@@ -2372,8 +2375,8 @@ static cudaError_t halves_inverse(float2* D, int64_t stride, float2* out, int n,
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
     // one Newton step
-    RCI_CUDA_TRY(launch_sg_split(A, true, n, stride, false, n, n, 3, c, w.D.f, w.D.e, nullptr, s, 5));
-    RCI_CUDA_TRY(launch_sg_split(X0, true, n, nn, true, n, n, 2, c, w.X.f, w.X.e, nullptr, s, 5));
+    RCI_CUDA_TRY(launch_sg_split(A, true, n, stride, false, n, n, 3, c, w.D.f, w.D.e, nullptr, s, 4));
+    RCI_CUDA_TRY(launch_sg_split(X0, true, n, nn, true, n, n, 2, c, w.X.f, w.X.e, nullptr, s, 4));
     SgJob r{};
     r.nseg = 1;
     r.seg[0] = SgSeg{w.D.f, w.D.e, w.X.f, w.X.e, 3, 2, 0, 0, 0, c};
@@ -2384,7 +2387,7 @@ static cudaError_t halves_inverse(float2* D, int64_t stride, float2* out, int n,
     r.sC = nn;
     r.batch = c;
     r.maxabs = maxabs;
-    RCI_CUDA_TRY(launch_sg_gemm(n, n, n, 1, &r, SG_HALF, status, wl, s));
+    RCI_CUDA_TRY(launch_sg_gemm(n, n, n, 1, &r, SG_SMALL, status, wl, s));
     halves_check_kernel<<<(unsigned)ceil_div(c, 128), 128, 0, s>>>(maxabs, n, c, failed, st32, status);
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());

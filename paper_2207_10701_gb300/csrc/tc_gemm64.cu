@@ -58,8 +58,10 @@ struct SgCfg {
   static constexpr int STAGES = 3 * STAGE + 2 * SG_STG_BYTES + 128 <= SG_SMEM_MAX ? 3 : 2;
   static constexpr uint32_t STG_OFF = STAGES * STAGE;
   static constexpr uint32_t BAR_OFF = STG_OFF + 2 * SG_STG_BYTES;
-  // A operands copied to tensor memory beside the accumulators where those leave four pairs of slots
-  static constexpr bool TS = 512 - ACC * NT >= 64;
+  // A operands copied to tensor memory beside the accumulators (four pairs of slots) where tiles are
+  // narrow: from 80 columns on an MMA is not bound by reading A from shared memory
+  static constexpr bool TS = NT <= 64;
+  static_assert(!TS || 512 - ACC * NT >= 64, "slots for A");
   static constexpr uint32_t SMEM = BAR_OFF + (2 * STAGES + 3) * 8 + 16;
   static_assert(SMEM <= SG_SMEM_MAX, "one CTA per SM beside the static shared memory");
   static_assert(SLOT % 128 == 0 && STG_OFF % 16 == 0 && NT % 16 == 0 && ACC * NT <= 512, "layout");
@@ -451,14 +453,12 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
         ok = agree(wait_warp(acc_full, (uint32_t)(ps & 1), abort_flag, p.wait_limit));
         if (!ok) break;
         f_after();
-        // join the accumulators of all the tile's slabs into registers, so that the next tile's MMAs
-        // start while the results are stored
         constexpr int SLABS = SG_NT / 16;
+        // narrow tiles: all slabs are joined into registers first, so that the next tile's MMAs start
+        // while the results are stored; wide ones (fewer digits, shorter epilogues) slab by slab
+        constexpr bool HOLD = SLABS <= 4;
         const int last = tl.nt >> 4;
-        double v[SLABS][4];
-#pragma unroll
-        for (int sb = 0; sb < SLABS; ++sb) {
-          if (sb >= last) break;
+        auto join = [&](int sb, double (&v)[4]) {
           float a[SG_ACC][4];
 #pragma unroll
           for (int w = 0; w < SG_ACC; ++w) tmem_ld4(tl_base + (uint32_t)(w * p.nt + 16 * sb + c4), a[w]);
@@ -480,12 +480,10 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
               else lo += n;
               u *= 256.f;
             }
-            v[sb][j] = scaled<8 * (SG_ACC > 3 ? SG_ACC - 3 : 0)>(hi, lo, ea, sh_eb[16 * sb + c4 + j]);
+            v[j] = scaled<8 * (SG_ACC > 3 ? SG_ACC - 3 : 0)>(hi, lo, ea, sh_eb[16 * sb + c4 + j]);
           }
-        }
-#pragma unroll
-        for (int sb = 0; sb < SLABS; ++sb) {
-          if (sb >= last) break;
+        };
+        auto store = [&](int sb, const double (&v)[4]) {
           // this thread's outputs of the slab, rows r and r + 32, column col; their C0 first
           const int col = tl.n0 + 16 * sb + (et & 15);
           const int r = et >> 4;
@@ -498,7 +496,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
           double* sp = reinterpret_cast<double*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES) +
                        (row * SG_STG_LD + c4) * 2 + part;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) sp[2 * j] = v[sb][j];
+          for (int j = 0; j < 4; ++j) sp[2 * j] = v[j];
           // the slab is whole; the other buffer's slab has been read by every warp before this
           asm volatile("bar.sync 1, %0;" ::"n"(32 * SG_EPI_WARPS) : "memory");
           const double2* sr = reinterpret_cast<const double2*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES);
@@ -524,6 +522,21 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
             }
           }
           ++slab;
+        };
+        if constexpr (HOLD) {
+          double v[SLABS][4];
+#pragma unroll
+          for (int sb = 0; sb < SLABS; ++sb)
+            if (sb < last) join(sb, v[sb]);
+#pragma unroll
+          for (int sb = 0; sb < SLABS; ++sb)
+            if (sb < last) store(sb, v[sb]);
+        } else {
+          for (int sb = 0; sb < last; ++sb) {
+            double v[4];
+            join(sb, v);
+            store(sb, v);
+          }
         }
         first = false;
         ++ps;
@@ -761,6 +774,7 @@ cudaError_t launch_sg_gemm(int M, int N, int K, int njob, const SgJob* jobs, SgD
   if (a.njob == 0) return cudaSuccess;
   switch (digits) {
     case SG_FULL: return launch_cfg<SgCfg<8, 7, 64>>(a, products, s);
+    case SG_SMALL: return launch_cfg<SgCfg<4, 4, 112>>(a, products, s);
     default: return launch_cfg<SgCfg<5, 5, 96>>(a, products, s);
   }
 }

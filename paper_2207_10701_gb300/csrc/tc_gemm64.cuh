@@ -57,8 +57,9 @@ struct SgJob {
 
 // Digit pairs kept: SG_FULL the 34 that count in FP64 (error about 2^-55 of the product of the
 // row's and the column's largest entries), SG_HALF the fifteen of weights down to 2^-32 (error
-// about 2^-36 of it: for corrections, and for residuals that are formed again).
-enum SgDigits { SG_FULL, SG_HALF };
+// about 2^-36 of it: for corrections, and for residuals that are formed again), SG_SMALL the ten
+// down to 2^-24 (2^-28).  They read seven, five and four digits.
+enum SgDigits { SG_FULL, SG_HALF, SG_SMALL };
 
 // One launch over one or two jobs of the same M, N, K (K <= SG_KMAX).  A wait that expires is
 // recorded as DEV_TIMEOUT in *status.
