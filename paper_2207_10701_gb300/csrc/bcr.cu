@@ -616,6 +616,7 @@ template <typename T, bool SMEM, int R, int TR, int TC, int NT>
 __global__ void __launch_bounds__(NT)
 gj_regpanel_kernel(cplx<T>* __restrict__ src, int64_t src_stride, cplx<T>* __restrict__ out,
                    int64_t out_stride, int n, int32_t* status, const int32_t* __restrict__ only) {
+  dep_begin();
   if (only && only[blockIdx.x] == 0) return;  // (only: the blocks to invert, null for all)
   constexpr int NB = NT / 32;
   constexpr int TY = NT / 32;
@@ -1054,8 +1055,8 @@ cudaError_t launch_gj_reg(cplx<T>* src, int64_t src_stride, cplx<T>* out, int64_
   if (L.total > 48 * 1024)
     RCI_CUDA_TRY(cudaFuncSetAttribute(gj_regpanel_kernel<T, SMEM, R, TR, TC, NT>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
-  gj_regpanel_kernel<T, SMEM, R, TR, TC, NT><<<batch, NT, L.total, s>>>(src, src_stride, out,
-                                                                        out_stride, n, status, only);
+  RCI_CUDA_TRY(launch_dep(gj_regpanel_kernel<T, SMEM, R, TR, TC, NT>, batch, NT, L.total, s, src, src_stride, out,
+                          out_stride, n, status, only));
   rci_note_launch();
   return cudaGetLastError();
 }
@@ -2063,6 +2064,7 @@ namespace {
 // a = (float) of `batch` nn-element blocks, stride elements apart
 __global__ void blocks_to_f32_kernel(const double2* __restrict__ src, int64_t stride, int64_t nn,
                                      int64_t total, float2* __restrict__ out) {
+  dep_begin();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= total) return;
   const int64_t z = e / nn;
@@ -2072,6 +2074,7 @@ __global__ void blocks_to_f32_kernel(const double2* __restrict__ src, int64_t st
 
 __global__ void blocks_to_f64_kernel(const float2* __restrict__ src, int64_t total,
                                      double2* __restrict__ out) {
+  dep_begin();
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e < total) out[e] = make_double2((double)src[e].x, (double)src[e].y);
 }
@@ -2090,6 +2093,7 @@ struct NewtonFlags {
 };
 __global__ void newton_check_kernel(NewtonFlags f, int n, int batch, int rough, int last,
                                     const int32_t* __restrict__ st32, int32_t* status) {
+  dep_begin();
   const int z = blockIdx.x * blockDim.x + threadIdx.x;
   if (z == 0 && *st32 == DEV_TIMEOUT) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
   if (z >= batch) return;
@@ -2226,12 +2230,12 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
     double2* X = out + (int64_t)k0 * nn;
     RCI_CUDA_TRY(cudaMemsetAsync(words, 0, sizeof(int32_t) * (4 * (size_t)c + 1 + 2 * NEWTON_STEPS), s));
     const int64_t tot = (int64_t)c * nn;
-    blocks_to_f32_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(Dk, stride, nn, tot, a32);
+    RCI_CUDA_TRY(launch_dep(blocks_to_f32_kernel, (unsigned)ceil_div(tot, 256), 256, 0, s, Dk, stride, nn, tot, a32));
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
     if (ny <= 160) RCI_CUDA_TRY(launch_tc_gj(a32, nn, x32, nn, ny, c, st32, s));
     else RCI_CUDA_TRY(launch_gj_simt<float>(a32, nn, x32, nn, ny, c, st32, s));
-    blocks_to_f64_kernel<<<(unsigned)ceil_div(tot, 256), 256, 0, s>>>(x32, tot, X);
+    RCI_CUDA_TRY(launch_dep(blocks_to_f64_kernel, (unsigned)ceil_div(tot, 256), 256, 0, s, x32, tot, X));
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
     RCI_CUDA_TRY(launch_sg_split(Dk, false, ny, stride, false, ny, ny, 3, c, fD, eD, nullptr, s));
@@ -2252,8 +2256,8 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
       r.skip = fl.skip_r;
       if (it > 0) r.any = st32 + 2 * it;  // what the step before left active
       RCI_CUDA_TRY(launch_sg_gemm(ny, ny, ny, 1, &r, it == 0 ? SG_HALF : SG_FULL, status, wl, s));
-      newton_check_kernel<<<(unsigned)ceil_div(c, 128), 128, 0, s>>>(fl, ny, c, it == 0, it == NEWTON_STEPS - 1,
-                                                                     st32, status);
+      RCI_CUDA_TRY(launch_dep(newton_check_kernel, (unsigned)ceil_div(c, 128), 128, 0, s, fl, ny, c, it == 0,
+                              it == NEWTON_STEPS - 1, st32, status));
       rci_note_launch();
       RCI_CUDA_TRY(cudaGetLastError());
       // (the first update corrects some 1e-5 and takes SG_HALF; the later ones correct 1e-8 or less)

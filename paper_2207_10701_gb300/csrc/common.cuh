@@ -1,6 +1,7 @@
 // Shared device helpers: complex arithmetic on float2/double2, status word, launch checks.
 #pragma once
 
+#include <utility>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -70,6 +71,37 @@ enum : int32_t { DEV_OK = 0, DEV_SINGULAR = 1, DEV_NONFINITE = 2, DEV_BADINPUT =
   } while (0)
 
 static inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// The FP64 factorisation is a chain of some forty launches a level, most of a few us.  They are launched
+// as dependents of the one before on the stream (programmatic stream serialisation): their blocks are
+// placed while that one drains, and the launch is off the chain.  Such a kernel starts with dep_begin(),
+// in all threads and before it reads or writes anything: it waits until the kernel before has completed
+// with its writes visible (and so, in turn, everything before that), then lets its own dependent be
+// placed.  New FP64 designs: 50 x 128 6.11 -> 5.40 ms, 500 x 160 39.0 -> 38.0.
+// The FP32 kernels are launched ordinarily: alone they gained under 1 %, and with four evaluations in
+// flight their waiting blocks kept the others off idle SMs (158 -> 152 evaluations/s at 500 x 160).
+__device__ __forceinline__ void dep_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Only for kernels that start with dep_begin().
+template <typename... P, typename... A>
+cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // reported here, not by a later call
+  return e;
+}
 
 // ---------------------------------------------------------------- device memory source
 // Where a grid and its factorisation get their device memory: cudaMalloc / cudaFree by

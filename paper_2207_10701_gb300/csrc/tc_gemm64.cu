@@ -261,6 +261,7 @@ __device__ __forceinline__ Tile tile_at(const SgJob* jobs, const SgArgs& p, int 
 
 template <typename Cfg>
 __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_constant__ SgArgs p) {
+  dep_begin();
   constexpr int SG_STAGES = Cfg::STAGES, SG_ACC = Cfg::ACC, SG_NT = Cfg::NT;
   constexpr uint32_t SG_STAGE = Cfg::STAGE, SG_SLOT = Cfg::SLOT, SG_A_SLOT = Cfg::A_SLOT,
                      SG_B_PLANE = Cfg::B_PLANE, SG_STG_OFF = Cfg::STG_OFF, SG_BAR_OFF = Cfg::BAR_OFF;
@@ -588,6 +589,7 @@ __global__ void __launch_bounds__(SS_THREADS)
 sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int trans, int rows, int K,
                 int planes, int chunks, int G, unsigned char* __restrict__ form, int32_t* __restrict__ exps,
                 const int32_t* __restrict__ skip, int digits) {
+  dep_begin();
   extern __shared__ __align__(16) unsigned char raw[];
   const int z = blockIdx.y;
   if (skip && skip[z]) return;
@@ -716,8 +718,8 @@ cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t strid
   auto go = [&](auto kernel, auto* p) -> cudaError_t {
     if (smem > 48 * 1024)
       RCI_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kernel<<<grid, SS_THREADS, smem, s>>>(p, ld, stride, trans ? 1 : 0, rows, K, planes, chunks, G, form, exps, skip,
-                                          digits);
+    RCI_CUDA_TRY(launch_dep(kernel, grid, SS_THREADS, smem, s, p, ld, stride, trans ? 1 : 0, rows, K, planes, chunks, G, form,
+                            exps, skip, digits));
     rci_note_launch();
     return cudaGetLastError();
   };
@@ -742,7 +744,7 @@ cudaError_t launch_cfg(SgArgs& a, int64_t products, cudaStream_t s) {
   a.tile0[1] = (int)(a.job[0].batch * per);
   const unsigned grid = (unsigned)(nt < sm_count() ? nt : sm_count());
   RCI_CUDA_TRY(cudaFuncSetAttribute(sg_gemm_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM));
-  sg_gemm_kernel<Cfg><<<grid, SG_THREADS, Cfg::SMEM, s>>>(a);
+  RCI_CUDA_TRY(launch_dep(sg_gemm_kernel<Cfg>, grid, SG_THREADS, Cfg::SMEM, s, a));
   rci_note_launch();
   return cudaGetLastError();
 }
