@@ -2052,7 +2052,7 @@ cudaError_t bcr_read_status(BcrHandle* h, int32_t* st, cudaStream_t s, double* g
 // block inverses as Newton iterations on an FP32 inverse, X <- X + X (I - D X), with those products:
 // the FP64 pipe does neither.  At ny = 160 a product takes 1.2 us of the whole GPU where the FP64
 // GEMM took 28, and an inverse of one block alone 0.4 ms where the FP64 Gauss-Jordan took 4.9: a
-// new design of 500 cells 404 -> 42 ms, of 50 cells (ny = 128) 54 -> 6.7 ms.
+// new design of 500 cells 404 -> 38 ms, of 50 cells (ny = 128) 54 -> 5.4 ms.
 // A block whose iteration does not contract (an FP32 inverse that resolves nothing, entries outside
 // the FP32 range, a singular block) goes to the FP64 Gauss-Jordan kernel, which also reports zero
 // pivots, so the factorisation accepts and refuses what it did.
