@@ -38,6 +38,8 @@ qform_tile_kernel(const double2* __restrict__ v, const double* __restrict__ lags
   __shared__ double lw[QT + U];
   __shared__ double red[QT];
   __shared__ double share[C];
+  // (the other blocks' shared memory may be written once they have started: the wait is below)
+  if constexpr (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;
   const int64_t tile = blockIdx.x / C;
   int64_t bi, bl;
@@ -74,6 +76,7 @@ qform_tile_kernel(const double2* __restrict__ v, const double* __restrict__ lags
   }
   if constexpr (C > 1) {
     cg::cluster_group cl = cg::this_cluster();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (t == 0) cl.map_shared_rank(share, 0)[rank] = red[0];
     cl.sync();
     if (rank != 0 || t != 0) return;
