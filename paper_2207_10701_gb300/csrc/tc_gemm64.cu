@@ -31,9 +31,12 @@
 // whole 256-byte row pieces.  The accumulators fill the tensor memory, so the next tile's MMAs
 // start when they have been joined into registers, under the stores.  SG_FULL copies a digit's A
 // windows to tensor memory once for all its pairs (tcgen05.cp): with A in shared memory an MMA
-// of 64 columns is bound by reading it.
+// of 64 columns is bound by reading it.  The slots are a ring: tensor memory orders a copy before the
+// MMAs that follow it, but not an MMA before the copy that overwrites its operand, so a slot's next
+// copy waits for a commit behind its MMAs (the three digits between keep the tensor cores busy).
 #include "tc_gemm64.cuh"
 #include "tc_gemm.cuh"
+#include "slot_ring.h"
 
 #include <cuda_bf16.h>
 
@@ -61,8 +64,8 @@ struct SgCfg {
   // A operands copied to tensor memory beside the accumulators (four pairs of slots) where tiles are
   // narrow: from 80 columns on an MMA is not bound by reading A from shared memory
   static constexpr bool TS = NT <= 64;
-  static_assert(!TS || 512 - ACC * NT >= 64, "slots for A");
-  static constexpr uint32_t SMEM = BAR_OFF + (2 * STAGES + 3) * 8 + 16;
+  static_assert(!TS || 512 - ACC * NT >= 16 * RING_SLOTS, "slots for A");
+  static constexpr uint32_t SMEM = BAR_OFF + (2 * STAGES + 3 + RING_SLOTS) * 8 + 16;
   static_assert(SMEM <= SG_SMEM_MAX, "one CTA per SM beside the static shared memory");
   static_assert(SLOT % 128 == 0 && STG_OFF % 16 == 0 && NT % 16 == 0 && ACC * NT <= 512, "layout");
 };
@@ -124,6 +127,16 @@ __device__ __forceinline__ bool wait_own(uint64_t* b, uint32_t parity) {
   const long long t0 = clock64();
   while (!bar_test(a, parity))
     if (clock64() - t0 > SG_OWN_WAIT) return false;
+  return true;
+}
+// bounded wait of one thread
+__device__ __forceinline__ bool wait_one(uint64_t* b, uint32_t parity, volatile int* abort_flag, long long limit) {
+  const uint32_t a = s32(b);
+  const long long t0 = clock64();
+  while (!bar_test(a, parity)) {
+    if (clock64() - t0 > limit) *abort_flag = 1;
+    if (*abort_flag) return false;
+  }
   return true;
 }
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint64_t* b) {
@@ -271,7 +284,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
   uint64_t* acc_full = empty + SG_STAGES;
   uint64_t* acc_empty = acc_full + 1;
   uint64_t* done_bar = acc_empty + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done_bar + 1);
+  uint64_t* slot_free = done_bar + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(slot_free + RING_SLOTS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   __shared__ SgJob jobs[2];
   __shared__ int32_t sh_eb[SG_NT];
@@ -287,6 +301,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
     bar_init(acc_full, 1);
     bar_init(acc_empty, SG_EPI_WARPS);
     bar_init(done_bar, 1);
+    for (int i = 0; i < RING_SLOTS; ++i) bar_init(&slot_free[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -385,10 +400,13 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
             const uint32_t more = c > 0 ? 1u : 0u;  // the first pair of an accumulator overwrites it
 #pragma unroll
             for (int i = 0; i < Cfg::DIG; ++i) {
-              // both windows of the digit, read once from shared memory for all its pairs (copies
-              // and MMAs of one thread run in order, so a slot is free when its turn comes again)
-              const uint32_t ta = tmem + (uint32_t)(SG_ACC * SG_NT) + 16u * (uint32_t)(i & 3);
+              // both windows of the digit, read once from shared memory for all its pairs
+              uint32_t ta = 0;
+              RingUse use{};
               if (Cfg::TS) {
+                use = ring_use((uint32_t)(it * Cfg::DIG + i));
+                ta = tmem + (uint32_t)(SG_ACC * SG_NT) + 16u * use.slot;
+                if (use.wait && !wait_one(&slot_free[use.slot], use.parity, abort_flag, p.wait_limit)) break;
                 copy_a(ta, a0 + i * SLOT16, dhi);
                 copy_a(ta + 8u, a0 + R16 + i * SLOT16, dhi);
               }
@@ -406,6 +424,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
                   mma_bf16(d, dhi, a0 + R16 + i * SLOT16, b0 + B16 + j * SLOT16, ineg, 1u);
                 }
               }
+              if (Cfg::TS) commit(&slot_free[use.slot]);
             }
             commit(&empty[st]);
           }
