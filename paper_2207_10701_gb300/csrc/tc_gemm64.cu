@@ -31,9 +31,9 @@
 // whole 256-byte row pieces.  The accumulators fill the tensor memory, so the next tile's MMAs
 // start when they have been joined into registers, under the stores.  SG_FULL copies a digit's A
 // windows to tensor memory once for all its pairs (tcgen05.cp): with A in shared memory an MMA
-// of 64 columns is bound by reading it.  The slots are a ring: tensor memory orders a copy before the
-// MMAs that follow it, but not an MMA before the copy that overwrites its operand, so a slot's next
-// copy waits for a commit behind its MMAs (the three digits between keep the tensor cores busy).
+// of 64 columns is bound by reading it.  Tensor memory orders a copy before the MMAs that follow it,
+// but not an MMA before the copy that overwrites its operand, so a slot's next copy waits for a commit
+// behind its MMAs (slot_ring.h).
 #include "tc_gemm64.cuh"
 #include "tc_gemm.cuh"
 #include "slot_ring.h"
@@ -64,8 +64,8 @@ struct SgCfg {
   // A operands copied to tensor memory beside the accumulators (four pairs of slots) where tiles are
   // narrow: from 80 columns on an MMA is not bound by reading A from shared memory
   static constexpr bool TS = NT <= 64;
-  static_assert(!TS || 512 - ACC * NT >= 16 * RING_SLOTS, "slots for A");
-  static constexpr uint32_t SMEM = BAR_OFF + (2 * STAGES + 3 + RING_SLOTS) * 8 + 16;
+  static_assert(!TS || (512 - ACC * NT >= 16 * RING_SLOTS && DIG == RING_DIGITS), "slots for A");
+  static constexpr uint32_t SMEM = BAR_OFF + (2 * STAGES + 3 + RING_GROUPS) * 8 + 16;
   static_assert(SMEM <= SG_SMEM_MAX, "one CTA per SM beside the static shared memory");
   static_assert(SLOT % 128 == 0 && STG_OFF % 16 == 0 && NT % 16 == 0 && ACC * NT <= 512, "layout");
 };
@@ -132,6 +132,7 @@ __device__ __forceinline__ bool wait_own(uint64_t* b, uint32_t parity) {
 // bounded wait of one thread
 __device__ __forceinline__ bool wait_one(uint64_t* b, uint32_t parity, volatile int* abort_flag, long long limit) {
   const uint32_t a = s32(b);
+  if (bar_test(a, parity)) return true;
   const long long t0 = clock64();
   while (!bar_test(a, parity)) {
     if (clock64() - t0 > limit) *abort_flag = 1;
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
   uint64_t* acc_empty = acc_full + 1;
   uint64_t* done_bar = acc_empty + 1;
   uint64_t* slot_free = done_bar + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(slot_free + RING_SLOTS);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(slot_free + RING_GROUPS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   __shared__ SgJob jobs[2];
   __shared__ int32_t sh_eb[SG_NT];
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
     bar_init(acc_full, 1);
     bar_init(acc_empty, SG_EPI_WARPS);
     bar_init(done_bar, 1);
-    for (int i = 0; i < RING_SLOTS; ++i) bar_init(&slot_free[i], 1);
+    for (int i = 0; i < RING_GROUPS; ++i) bar_init(&slot_free[i], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -401,12 +402,12 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
 #pragma unroll
             for (int i = 0; i < Cfg::DIG; ++i) {
               // both windows of the digit, read once from shared memory for all its pairs
-              uint32_t ta = 0;
-              RingUse use{};
+              const uint32_t ta = tmem + (uint32_t)(SG_ACC * SG_NT) + 16u * ring_slot(i);
               if (Cfg::TS) {
-                use = ring_use((uint32_t)(it * Cfg::DIG + i));
-                ta = tmem + (uint32_t)(SG_ACC * SG_NT) + 16u * use.slot;
-                if (use.wait && !wait_one(&slot_free[use.slot], use.parity, abort_flag, p.wait_limit)) break;
+                const int g = ring_group(i);
+                if (ring_first(i) && ring_waits(g, it) &&
+                    !wait_one(&slot_free[ring_wait_group(g)], ring_parity(g, it), abort_flag, p.wait_limit))
+                  break;
                 copy_a(ta, a0 + i * SLOT16, dhi);
                 copy_a(ta + 8u, a0 + R16 + i * SLOT16, dhi);
               }
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
                   mma_bf16(d, dhi, a0 + R16 + i * SLOT16, b0 + B16 + j * SLOT16, ineg, 1u);
                 }
               }
-              if (Cfg::TS) commit(&slot_free[use.slot]);
+              if (Cfg::TS && ring_last(i)) commit(&slot_free[ring_group(i)]);
             }
             commit(&empty[st]);
           }
