@@ -460,8 +460,9 @@ rci_status rci_block_inverse(const void* src, void* out, int64_t n, int64_t batc
  * kernel: 0 = the factorisation's dispatch; 1 = tensor cores (3xTF32 tcgen05), operands
  * staged through registers into shared memory; 2 = tensor cores fed by TMA with the A
  * operand in tensor memory (needs 2 <= N <= 160 and even, 16-byte aligned A, B, C, C0, even
- * leading dimensions and, for batch > 1, even positive sA, sB); 3 = SIMT.  Kernels 1 and 2
- * are FP32 only; the SIMT kernel (3, and 0 where it dispatches there: FP64, or batches too
+ * leading dimensions and, for batch > 1, even positive sA, sB); 3 = SIMT; 4 = the digit split
+ * of FP64 on the tensor cores (FP64 only, K <= 248, alpha = 1 or -1, beta = 1 with a C0; allocates
+ * its operands' split forms).  Kernels 1 and 2 are FP32 only; the SIMT kernel (3, and 0 where it dispatches there: FP64, or batches too
  * small to fill the GPU) has no form with both operands transposed.  Synchronises `stream` (cudaStream_t or NULL) and allocates a 4-byte status
  * word.  Errors: EINVAL (sizes, a kernel that does not apply), ETIMEOUT, ECUDA. */
 rci_status rci_cgemm_batched(int64_t M, int64_t N, int64_t K, int32_t ta, int32_t tb,

@@ -3206,6 +3206,32 @@ cudaError_t bcr_gemm(int M, int N, int K, bool ta, bool tb, double alpha, const 
                      int batch, int prec, int kernel, int32_t* status, cudaStream_t s) {
   if (prec == RCI_FP64) {
     if (kernel == 1 || kernel == 2) return cudaErrorInvalidValue;
+    if (kernel == 4) {
+      if (K > SG_KMAX || (alpha != 1.0 && alpha != -1.0) || (C0 && beta != 1.0)) return cudaErrorInvalidValue;
+      const size_t fa = batch * sg_form_bytes(M, K, 3), fb = batch * sg_form_bytes(N, K, 2);
+      const size_t ea = sizeof(int32_t) * batch * sg_form_exps(M), eb = sizeof(int32_t) * batch * sg_form_exps(N);
+      unsigned char* w = nullptr;
+      RCI_CUDA_TRY(cudaMalloc(&w, fa + fb + ea + eb));
+      unsigned char* wb = w + fa;
+      int32_t *xa = reinterpret_cast<int32_t*>(wb + fb), *xb = reinterpret_cast<int32_t*>(wb + fb + ea);
+      SgJob j{};
+      j.nseg = 1;
+      j.seg[0] = SgSeg{w, xa, wb, xb, 3, 2, 0, 0, 0, batch};
+      j.neg = alpha < 0;
+      j.C0 = (const double2*)C0;
+      j.ldc0 = ldc0;
+      j.sC0 = sC0;
+      j.C = (double2*)C;
+      j.ldc = ldc;
+      j.sC = sC;
+      j.batch = batch;
+      cudaError_t e = launch_sg_split(A, false, lda, sA, ta, M, K, 3, batch, w, xa, nullptr, s);
+      if (e == cudaSuccess) e = launch_sg_split(B, false, ldb, sB, !tb, N, K, 2, batch, wb, xb, nullptr, s);
+      if (e == cudaSuccess) e = launch_sg_gemm(M, N, K, 1, &j, SG_FULL, status, tc_wait_limit(), s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      cudaFree(w);
+      return e;
+    }
     const cplx<double> al{alpha, 0.0}, be{beta, 0.0};
     return gemm<double>(M, N, K, ta, tb, al, (const double2*)A, lda, sA, (const double2*)B, ldb,
                         sB, be, (const double2*)C0, ldc0, sC0, (double2*)C, ldc, sC, batch, s);

@@ -1517,7 +1517,8 @@ rci_status rci_cgemm_batched(int64_t M, int64_t N, int64_t K, int32_t ta, int32_
                              int32_t prec, int32_t kernel, void* stream) {
   const int64_t lim = 1 << 20;
   if (!A || !B || !C || M < 1 || N < 1 || K < 1 || M > lim || N > lim || K > lim || batch < 1 ||
-      batch > 65535 || kernel < 0 || kernel > 3 || (prec != RCI_FP64 && prec != RCI_FP32_REFINE))
+      batch > 65535 || kernel < 0 || kernel > (prec == RCI_FP64 ? 4 : 3) ||
+      (prec != RCI_FP64 && prec != RCI_FP32_REFINE))
     return RCI_EINVAL;
   if (!std::isfinite(alpha) || !std::isfinite(beta)) return RCI_EINVAL;
   const int64_t am = ta ? K : M, ak = ta ? M : K, bk = tb ? N : K, bn = tb ? K : N;

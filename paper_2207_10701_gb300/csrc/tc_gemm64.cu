@@ -4,14 +4,24 @@
 // (cuBLAS, 8192^3).  Each operand row (terms k along it) is scaled by a power of two and cut
 // into seven signed digits of eight bits (Ozaki's error-free splitting, here with fixed-point
 // digits and one exponent per row): x = 2^(e - 7) sum_s d_s 2^(-8 s), s = 0 .. 6, |d_s| <= 128,
-// exact to 2^(e - 56).  Digits are exact in bf16, a product of two digits is at most 2^14 and
-// 2 K <= 496 of them sum to less than 2^23, so an FP32 accumulator holds the sum of a digit pair
-// exactly; pairs (i, j) of equal weight i + j share an accumulator.  SG_FULL keeps the 34 pairs
+// exact to 2^(e - 56).  Digits are exact in bf16, and pairs (i, j) of equal weight i + j share an
+// FP32 accumulator, which is exact while the sums in it stay within 2^24.  SG_FULL keeps the 34 pairs
 // with i + j <= 7 in seven accumulators, the two lowest weights sharing one.  Fewer do not do:
 // on blocks like the solver's (dominant diagonals), the error of I - D D^-1 at n = 160 against
 // 113-bit sums is 2.7e-17 with them, 4.9e-17 with the FP64 FMA loop, 1.6e-16 when the weights
 // 5 to 7 share an accumulator and 5.8e-16 without i + j = 7.  Per output the accumulators are
 // joined in 64-bit integers and rounded once to FP64.
+//
+// Exactness.  A digit product is at most 2^14 and weight w sums 2 K (w + 1) of them, so whatever the
+// digits, weight 4 stays within 2^24 up to K = 102 only.  Digits of mixed sign stay far below it.  With
+// T the sum of the squares of a row's digits 0 .. 4, no partial sum of the weights 0 .. 4 exceeds
+// (T_a T_b)^(1/2) (Cauchy-Schwarz over the pairs of a weight); digits spread evenly give T = 54600 K,
+// 8.7e6 at K = 160 and 13.5e6 at K = 248, where 2^24 = 16.8e6 is allowed.  For SG_FULL the split marks
+// the groups of rows with a row of too large T, and a tile that meets one makes a pass with an epilogue
+// of its own for every 96 terms, for which the first bound holds.  The weights from 5 on may round: by
+// 2^-43 of the product of the row's and the column's largest entries if all digits agree, where the
+// bound of the FP64 FMA loop is 2^-36.  So may the accumulators of the shorter forms, by 2^-23: their
+// products are corrections, or residuals that are formed again.
 //
 // Measured, 608 products of 160^3: SG_FULL 710 us (1.17 us a product, 28 TFLOP/s of FP64 work; the
 // FP64 GEMM takes 28 us a product; 897 us with A in shared memory and an epilogue that the MMAs
@@ -54,6 +64,7 @@ template <int W_, int ACC_, int NT_>
 struct SgCfg {
   static constexpr int W = W_, ACC = ACC_, NT = NT_;
   static constexpr int DIG = W < SG_SLICES ? W : SG_SLICES;      // digits read
+  static constexpr bool MARKS = DIG == SG_SLICES;                // passes for marked rows
   static constexpr uint32_t A_SLOT = 3 * SG_ROWS * 32;           // planes r, i, -r
   static constexpr uint32_t B_PLANE = NT * 32;
   static constexpr uint32_t SLOT = A_SLOT + 2 * B_PLANE;
@@ -72,6 +83,8 @@ struct SgCfg {
 constexpr uint32_t SG_LBO = 128, SG_SBO = 256;
 constexpr int32_t SG_EXP_NONFINITE = 0x7fffffff;
 constexpr long long SG_OWN_WAIT = 4000000000LL;
+constexpr int SG_PART = 6;               // chunks whose sums of weight <= 4 are exact for any digits
+static_assert(5 * 2 * 16 * SG_PART * (1 << 14) <= 1 << 24, "");
 
 struct SgArgs {
   int M, N, K;
@@ -248,9 +261,9 @@ __device__ __forceinline__ void f_before() { asm volatile("tcgen05.fence::before
 __device__ __forceinline__ void f_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // ---------------------------------------------------------------- passes of a CTA
-// tile -> job, product, row tile, column tile; each tile makes one pass per segment it takes
-// part in, every pass a full accumulation and epilogue of its own (the segments' operands have
-// their own exponents).
+// tile -> job, product, row tile, column tile; each tile makes one pass (or several, see above) per
+// segment it takes part in, every pass a full accumulation and epilogue of its own (the segments'
+// operands have their own exponents).
 struct Tile {
   int j, z, i0, n0, nt;  // nt: the tile's columns rounded up to 16
   bool run, v[2];
@@ -271,6 +284,21 @@ __device__ __forceinline__ Tile tile_at(const SgJob* jobs, const SgArgs& p, int 
   r.v[0] = r.run && r.z >= jb.seg[0].zlo && r.z < jb.seg[0].zhi;
   r.v[1] = r.run && jb.nseg > 1 && r.z >= jb.seg[1].zlo && r.z < jb.seg[1].zhi;
   return r;
+}
+
+// The marks of a tile's row groups, one per lane; where any lane has one, segment g takes a pass for
+// every SG_PART chunks.  (They are voted on when the first SG_PART chunks are through, so that the loads
+// are not waited for.)
+__device__ __forceinline__ int32_t marks_of(const SgJob& jb, const SgArgs& p, const Tile& t, int g) {
+  if (p.chunks <= SG_PART) return 0;
+  const int lane = threadIdx.x & 31;
+  const SgSeg& sg = jb.seg[g];
+  if (lane < SG_ROWS / 8) {
+    const int a = (t.i0 >> 3) + lane;
+    return a < p.GA ? sg.eA[(int64_t)(t.z + sg.zA) * (p.GA * 9) + p.GA * 8 + a] : 0;
+  }
+  const int b = (t.n0 >> 3) + lane - SG_ROWS / 8;
+  return lane - SG_ROWS / 8 < t.nt / 8 && b < p.GB ? sg.eB[(int64_t)(t.z + sg.zB) * (p.GB * 9) + p.GB * 8 + b] : 0;
 }
 
 template <typename Cfg>
@@ -349,7 +377,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
           off = SG_A_SLOT + (uint32_t)(lane - 3) * SG_B_PLANE;
           bytes = bb;
         }
-        for (int c = 0; c < p.chunks; ++c, ++it) {
+        for (int c = 0; c < p.chunks; ++c, ++it) {  // (the passes of a segment one after the other)
           const int st = it % SG_STAGES;
           if (it >= SG_STAGES &&
               !wait_warp(&empty[st], (uint32_t)((it / SG_STAGES - 1) & 1), abort_flag, p.wait_limit)) {
@@ -382,15 +410,26 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
       const Tile tl = tile_at(jobs, p, t);
       for (int g = 0; g < 2 && ok; ++g) {
         if (!tl.v[g]) continue;
-        if (ps >= 1 && !wait_warp(acc_empty, (uint32_t)((ps - 1) & 1), abort_flag, p.wait_limit)) {
-          ok = false;
-          break;
-        }
-        f_after();
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(tl.nt >> 3) << 17) |
                                ((uint32_t)(128 >> 4) << 24);
         const uint32_t ineg = idesc | (1u << 13);  // -A
-        for (int c = 0; c < p.chunks; ++c, ++it) {
+        const int32_t mark = Cfg::MARKS ? marks_of(jobs[tl.j], p, tl, g) : 0;
+        int len = p.chunks;  // chunks of a pass
+        for (int c = 0, cp = 0; c < p.chunks; ++c, ++cp, ++it) {
+          if (Cfg::MARKS && c == SG_PART && __any_sync(0xffffffffu, mark != 0)) len = SG_PART;
+          if (cp == len) {
+            if (elect_one()) commit(acc_full);
+            __syncwarp();
+            ++ps;
+            cp = 0;
+          }
+          if (cp == 0) {
+            if (ps >= 1 && !wait_warp(acc_empty, (uint32_t)((ps - 1) & 1), abort_flag, p.wait_limit)) {
+              ok = false;
+              break;
+            }
+            f_after();
+          }
           const int st = it % SG_STAGES;
           if (!wait_warp(&full[st], (uint32_t)((it / SG_STAGES) & 1), abort_flag, p.wait_limit)) {
             ok = false;
@@ -398,7 +437,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
           }
           if (elect_one()) {
             const uint32_t a0 = dlo + ((smb + (uint32_t)st * SG_STAGE) >> 4), b0 = a0 + A16;
-            const uint32_t more = c > 0 ? 1u : 0u;  // the first pair of an accumulator overwrites it
+            const uint32_t more = cp > 0 ? 1u : 0u;  // the first pair of an accumulator overwrites it
 #pragma unroll
             for (int i = 0; i < Cfg::DIG; ++i) {
               // both windows of the digit, read once from shared memory for all its pairs
@@ -460,107 +499,113 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
       uint32_t big = 0;  // largest high word of |re|, |im|
       for (int g = 0; g < 2 && ok; ++g) {
         if (!tl.v[g]) continue;
-        const SgSeg& sg = jb.seg[g];
-        const int32_t* eA = sg.eA + (int64_t)(tl.z + sg.zA) * (p.GA * 8);
-        const int32_t* eB = sg.eB + (int64_t)(tl.z + sg.zB) * (p.GB * 8);
-        const int ea = tl.i0 + row < p.M ? eA[tl.i0 + row] : 0;
-        const double2* C0 = first ? (jb.C0 ? jb.C0 + tl.z * jb.sC0 : nullptr) : jb.C + tl.z * jb.sC;
-        const int64_t ldc0 = first ? jb.ldc0 : jb.ldc;
-        const bool eye = first && jb.identity;
-        // the columns' exponents (the threads that read the last pass's are past a barrier since)
-        if (et < p.nt) sh_eb[et] = tl.n0 + et < p.N ? eB[tl.n0 + et] : 0;
-        double2* C = jb.C + tl.z * jb.sC;
-        // the eight warps go on or give up together (they meet at barriers below)
-        ok = agree(wait_warp(acc_full, (uint32_t)(ps & 1), abort_flag, p.wait_limit));
-        if (!ok) break;
-        f_after();
-        constexpr int SLABS = SG_NT / 16;
-        // narrow tiles: all slabs are joined into registers first, so that the next tile's MMAs start
-        // while the results are stored; wide ones (fewer digits, shorter epilogues) slab by slab
-        constexpr bool HOLD = SLABS <= 4;
-        const int last = tl.nt >> 4;
-        auto join = [&](int sb, double (&v)[4]) {
-          float a[SG_ACC][4];
+        const int32_t mark = Cfg::MARKS ? marks_of(jb, p, tl, g) : 0;
+        int len = p.chunks;
+        for (int pass = 0; pass < p.chunks; pass += len) {
+          big = 0;  // (of the last pass, which leaves the output)
+          const SgSeg& sg = jb.seg[g];
+          const int32_t* eA = sg.eA + (int64_t)(tl.z + sg.zA) * (p.GA * 9);
+          const int32_t* eB = sg.eB + (int64_t)(tl.z + sg.zB) * (p.GB * 9);
+          const int ea = tl.i0 + row < p.M ? eA[tl.i0 + row] : 0;
+          const double2* C0 = first ? (jb.C0 ? jb.C0 + tl.z * jb.sC0 : nullptr) : jb.C + tl.z * jb.sC;
+          const int64_t ldc0 = first ? jb.ldc0 : jb.ldc;
+          const bool eye = first && jb.identity;
+          // the columns' exponents (the threads that read the last pass's are past a barrier since)
+          if (et < p.nt) sh_eb[et] = tl.n0 + et < p.N ? eB[tl.n0 + et] : 0;
+          double2* C = jb.C + tl.z * jb.sC;
+          // the epilogue warps go on or give up together (they meet at barriers below)
+          ok = agree(wait_warp(acc_full, (uint32_t)(ps & 1), abort_flag, p.wait_limit));
+          if (!ok) break;
+          f_after();
+          if (Cfg::MARKS && __any_sync(0xffffffffu, mark != 0)) len = SG_PART;
+          constexpr int SLABS = SG_NT / 16;
+          // narrow tiles: all slabs are joined into registers first, so that the next tile's MMAs start
+          // while the results are stored; wide ones (fewer digits, shorter epilogues) slab by slab
+          constexpr bool HOLD = SLABS <= 4;
+          const int last = tl.nt >> 4;
+          auto join = [&](int sb, double (&v)[4]) {
+            float a[SG_ACC][4];
 #pragma unroll
-          for (int w = 0; w < SG_ACC; ++w) tmem_ld4(tl_base + (uint32_t)(w * p.nt + 16 * sb + c4), a[w]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (sb == last - 1) {
-            f_before();
-            __syncwarp();
-            if (lane == 0) bar_arrive(acc_empty);
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            // accumulator w in units of 2^(-8 w), joined in units of 2^(-8 (ACC - 1))
-            long long hi = 0, lo = 0;
-            float u = 1.f;
-#pragma unroll
-            for (int w = 0; w < SG_ACC; ++w) {
-              const long long n = (long long)__float2int_rn(a[w][j] * u) << (8 * ((w < 3 ? 2 : SG_ACC - 1) - w));
-              if (w < 3) hi += n;
-              else lo += n;
-              u *= 256.f;
+            for (int w = 0; w < SG_ACC; ++w) tmem_ld4(tl_base + (uint32_t)(w * p.nt + 16 * sb + c4), a[w]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (sb == last - 1) {
+              f_before();
+              __syncwarp();
+              if (lane == 0) bar_arrive(acc_empty);
             }
-            v[j] = scaled<8 * (SG_ACC > 3 ? SG_ACC - 3 : 0)>(hi, lo, ea, sh_eb[16 * sb + c4 + j]);
-          }
-        };
-        auto store = [&](int sb, const double (&v)[4]) {
-          // this thread's outputs of the slab, rows r and r + 32, column col; their C0 first
-          const int col = tl.n0 + 16 * sb + (et & 15);
-          const int r = et >> 4;
-          double2 c0[2];
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int gr = tl.i0 + r + 32 * i;
-            c0[i] = (C0 && gr < p.M && col < p.N) ? C0[(int64_t)gr * ldc0 + col] : make_double2(0.0, 0.0);
-          }
-          double* sp = reinterpret_cast<double*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES) +
-                       (row * SG_STG_LD + c4) * 2 + part;
+            for (int j = 0; j < 4; ++j) {
+              // accumulator w in units of 2^(-8 w), joined in units of 2^(-8 (ACC - 1))
+              long long hi = 0, lo = 0;
+              float u = 1.f;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) sp[2 * j] = v[j];
-          // the slab is whole; the other buffer's slab has been read by every warp before this
-          asm volatile("bar.sync 1, %0;" ::"n"(32 * SG_EPI_WARPS) : "memory");
-          const double2* sr = reinterpret_cast<const double2*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES);
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const int gr = tl.i0 + r + 32 * i;
-            if (gr < p.M && col < p.N) {
-              double2 o = sr[(r + 32 * i) * SG_STG_LD + (et & 15)];
-              if (neg) {
-                o.x = -o.x;
-                o.y = -o.y;
+              for (int w = 0; w < SG_ACC; ++w) {
+                const long long n = (long long)__float2int_rn(a[w][j] * u) << (8 * ((w < 3 ? 2 : SG_ACC - 1) - w));
+                if (w < 3) hi += n;
+                else lo += n;
+                u *= 256.f;
               }
-              if (eye) {
-                if (gr == col) o.x += 1.0;
-              } else if (C0) {
-                o.x += c0[i].x;
-                o.y += c0[i].y;
+              v[j] = scaled<8 * (SG_ACC > 3 ? SG_ACC - 3 : 0)>(hi, lo, ea, sh_eb[16 * sb + c4 + j]);
+            }
+          };
+          auto store = [&](int sb, const double (&v)[4]) {
+            // this thread's outputs of the slab, rows r and r + 32, column col; their C0 first
+            const int col = tl.n0 + 16 * sb + (et & 15);
+            const int r = et >> 4;
+            double2 c0[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const int gr = tl.i0 + r + 32 * i;
+              c0[i] = (C0 && gr < p.M && col < p.N) ? C0[(int64_t)gr * ldc0 + col] : make_double2(0.0, 0.0);
+            }
+            double* sp = reinterpret_cast<double*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES) +
+                         (row * SG_STG_LD + c4) * 2 + part;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sp[2 * j] = v[j];
+            // the slab is whole; the other buffer's slab has been read by every warp before this
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * SG_EPI_WARPS) : "memory");
+            const double2* sr = reinterpret_cast<const double2*>(stg + (uint32_t)(slab & 1) * SG_STG_BYTES);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const int gr = tl.i0 + r + 32 * i;
+              if (gr < p.M && col < p.N) {
+                double2 o = sr[(r + 32 * i) * SG_STG_LD + (et & 15)];
+                if (neg) {
+                  o.x = -o.x;
+                  o.y = -o.y;
+                }
+                if (eye) {
+                  if (gr == col) o.x += 1.0;
+                } else if (C0) {
+                  o.x += c0[i].x;
+                  o.y += c0[i].y;
+                }
+                if (jb.C32) jb.C32[tl.z * jb.sC + (int64_t)gr * jb.ldc + col] = make_float2((float)o.x, (float)o.y);
+                else C[(int64_t)gr * jb.ldc + col] = o;
+                big = max(big, max((uint32_t)__double2hiint(o.x) & 0x7fffffffu,
+                                   (uint32_t)__double2hiint(o.y) & 0x7fffffffu));
               }
-              if (jb.C32) jb.C32[tl.z * jb.sC + (int64_t)gr * jb.ldc + col] = make_float2((float)o.x, (float)o.y);
-              else C[(int64_t)gr * jb.ldc + col] = o;
-              big = max(big, max((uint32_t)__double2hiint(o.x) & 0x7fffffffu,
-                                 (uint32_t)__double2hiint(o.y) & 0x7fffffffu));
+            }
+            ++slab;
+          };
+          if constexpr (HOLD) {
+            double v[SLABS][4];
+#pragma unroll
+            for (int sb = 0; sb < SLABS; ++sb)
+              if (sb < last) join(sb, v[sb]);
+#pragma unroll
+            for (int sb = 0; sb < SLABS; ++sb)
+              if (sb < last) store(sb, v[sb]);
+          } else {
+            for (int sb = 0; sb < last; ++sb) {
+              double v[4];
+              join(sb, v);
+              store(sb, v);
             }
           }
-          ++slab;
-        };
-        if constexpr (HOLD) {
-          double v[SLABS][4];
-#pragma unroll
-          for (int sb = 0; sb < SLABS; ++sb)
-            if (sb < last) join(sb, v[sb]);
-#pragma unroll
-          for (int sb = 0; sb < SLABS; ++sb)
-            if (sb < last) store(sb, v[sb]);
-        } else {
-          for (int sb = 0; sb < last; ++sb) {
-            double v[4];
-            join(sb, v);
-            store(sb, v);
-          }
+          first = false;
+          ++ps;
         }
-        first = false;
-        ++ps;
       }
       if (ok && jb.maxabs && tl.run) {
         const uint32_t wm = __reduce_max_sync(0xffffffffu, big);
@@ -587,7 +632,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sg_gemm_kernel(const __grid_con
 // thread takes eight consecutive terms of a row: the value as a 56-bit fixed-point integer, its
 // balanced base-256 digits as the bytes of q + 0x808080808080, turned into floats by a byte
 // permute and one FMA each, and stored as 16-byte core-matrix rows (16 threads cover 256
-// contiguous bytes).  Bound by the integer issue rate: about 30 instructions per real.
+// contiguous bytes).  Bound by the integer issue rate: about 34 instructions per real.
 constexpr int SS_THREADS = 256;
 
 __device__ __forceinline__ long long fixed56(double x, int e) {
@@ -608,14 +653,15 @@ template <typename T, int SS_ROWS>
 __global__ void __launch_bounds__(SS_THREADS)
 sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int trans, int rows, int K,
                 int planes, int chunks, int G, unsigned char* __restrict__ form, int32_t* __restrict__ exps,
-                const int32_t* __restrict__ skip, int digits) {
+                const int32_t* __restrict__ skip, int digits, int limit) {
   dep_begin();
   extern __shared__ __align__(16) unsigned char raw[];
   const int z = blockIdx.y;
   if (skip && skip[z]) return;
   const int Kp = chunks * 16, LD = Kp + 1;
   cplx<T>* t = reinterpret_cast<cplx<T>*>(raw);
-  __shared__ int re[SS_ROWS];
+  __shared__ int re[SS_ROWS], energy[SS_ROWS];
+  if (threadIdx.x < SS_ROWS) energy[threadIdx.x] = 0;
   const int r0 = blockIdx.x * SS_ROWS;
   const cplx<T>* S = src + (int64_t)z * stride;
   if (!trans) {
@@ -646,13 +692,14 @@ sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int
       const int e = m == 0x7ff ? SG_EXP_NONFINITE : (m == 0 ? 0 : m - 1022);
       re[r] = e;
       const int g = (r0 + r) >> 3;
-      if (g < G) exps[(int64_t)z * (G * 8) + r0 + r] = e;
+      if (g < G) exps[(int64_t)z * (G * 9) + r0 + r] = e;
     }
   }
   __syncthreads();
   const int64_t fbytes = (int64_t)chunks * SG_SLICES * planes * G * 256;
   unsigned char* F = form + (int64_t)z * fbytes;
   const int g0 = r0 >> 3;
+  int en = 0;  // this thread's squares of the digits 0 .. 4, all of one row
   // item: row-in-group (8) | term half (2) | group (2) | part (2) | chunk
   for (int it = threadIdx.x; it < chunks * 4 * SS_ROWS; it += SS_THREADS) {
     constexpr int GL = SS_ROWS == 16 ? 1 : 0;  // bits of the group
@@ -666,6 +713,13 @@ sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int
     for (int j = 0; j < 8; ++j) {
       const cplx<T> v = t[r * LD + c * 16 + kc * 8 + j];
       q[j] = (e == SG_EXP_NONFINITE ? 0 : fixed56((double)(part ? v.y : v.x), e)) + 0x808080808080LL;
+    }
+    if (limit != 0) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int d0 = (int)(q[j] >> 48), d = (int)((uint32_t)(q[j] >> 16) ^ 0x80808080u);
+        en = __dp4a(d, d, en) + d0 * d0;
+      }
     }
     unsigned char* out = F + ((int64_t)c * SG_SLICES * planes * G + g0 + gg) * 256 + kc * 128 + rr * 16;
     float w = 1.f;
@@ -703,6 +757,16 @@ sg_split_kernel(const cplx<T>* __restrict__ src, int64_t ld, int64_t stride, int
       w *= 0.00390625f;
     }
   }
+  // the marks of the row groups, behind the exponents
+  if (limit != 0) {
+    atomicAdd(&energy[((threadIdx.x >> 4) % (SS_ROWS / 8)) * 8 + (threadIdx.x & 7)], en);
+    __syncthreads();
+  }
+  if (threadIdx.x < SS_ROWS / 8 && g0 + (int)threadIdx.x < G) {
+    int m = 0;
+    for (int r = 0; r < 8; ++r) m = max(m, energy[8 * threadIdx.x + r]);
+    exps[(int64_t)z * (G * 9) + G * 8 + g0 + threadIdx.x] = m > limit ? 1 : 0;
+  }
 }
 
 int sm_count() {
@@ -735,11 +799,17 @@ cudaError_t launch_sg_split(const void* src, bool f32, int64_t ld, int64_t strid
   const int per = few ? 8 : 16;
   const size_t smem = (size_t)per * (chunks * 16 + 1) * (f32 ? sizeof(float2) : sizeof(double2));
   const dim3 grid((unsigned)ceil_div(rows, per), (unsigned)batch);
+  // Squares of a row's digits 0 .. 4 up to which it is not marked; 0: no marks.  Up to K = 160 the left
+  // operands' limit allows for any digits in the right ones, which then need none (the limit is 10.7e6
+  // at K = 160, where digits spread evenly give 8.7e6).
+  int limit = 0;
+  if (digits == SG_SLICES && chunks > SG_PART)
+    limit = K > 160 ? 1 << 24 : planes == 3 ? (int)((1LL << 48) / (5LL * 2 * K << 14)) : 0;
   auto go = [&](auto kernel, auto* p) -> cudaError_t {
     if (smem > 48 * 1024)
       RCI_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RCI_CUDA_TRY(launch_dep(kernel, grid, SS_THREADS, smem, s, p, ld, stride, trans ? 1 : 0, rows, K, planes, chunks, G, form,
-                            exps, skip, digits));
+                            exps, skip, digits, limit));
     rci_note_launch();
     return cudaGetLastError();
   };

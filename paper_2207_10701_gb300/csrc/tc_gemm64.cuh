@@ -4,15 +4,15 @@
 
 #include "common.cuh"
 
-// Most terms K of a product (the sum of 2 K products of digits has to stay below 2^23).
+// Most terms K of a product (2 K digit products stay below 2^23, for which the accumulators are joined).
 constexpr int SG_KMAX = 248;
 constexpr int SG_SLICES = 7;
 
 // Split form of one R x K complex operand (K contiguous terms per row): bytes of the digits with
 // `planes` planes (3: usable as the left or the right operand, 2: right operand only) and number
-// of row exponents.
+// of words for the row exponents and a mark for each group of eight rows.
 size_t sg_form_bytes(int rows, int K, int planes);
-inline int sg_form_exps(int rows) { return (int)ceil_div(rows, 8) * 8; }
+inline int sg_form_exps(int rows) { return (int)ceil_div(rows, 8) * 9; }
 
 // Split `batch` operands: row r, term k of operand z is src[z][r][k] (trans == false) or
 // src[z][k][r] (trans), row-major with leading dimension ld and `stride` complex elements between
@@ -56,7 +56,8 @@ struct SgJob {
 };
 
 // Digit pairs kept: SG_FULL the 34 that count in FP64 (error about 2^-55 of the product of the
-// row's and the column's largest entries), SG_HALF the fifteen of weights down to 2^-32 (error
+// row's and the column's largest entries, for digits of mixed sign; entries below 2^-56 of their row's
+// largest count as zero, and so do subnormals), SG_HALF the fifteen of weights down to 2^-32 (error
 // about 2^-36 of it: for corrections, and for residuals that are formed again), SG_SMALL the ten
 // down to 2^-24 (2^-28).  They read seven, five and four digits.
 enum SgDigits { SG_FULL, SG_HALF, SG_SMALL };

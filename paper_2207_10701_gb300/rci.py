@@ -467,7 +467,8 @@ def cgemm_batched(A, B, C0=None, alpha: float = 1.0, beta: float = 0.0, ta: bool
     GEMM kernels (rci_cgemm_batched): CUDA tensors [batch, rows, cols] of complex64 or
     complex128 whose rows are contiguous (any row and batch strides); op = transpose when ta
     / tb.  kernel 0 = the factorisation's dispatch, 1 = tensor cores with register-staged
-    operands, 2 = tensor cores fed by TMA, 3 = SIMT.  Returns C (`out` when given)."""
+    operands, 2 = tensor cores fed by TMA, 3 = SIMT, 4 = the FP64 digit split.  Returns C
+    (`out` when given)."""
     torch = _torch()
     for t in (A, B) + ((C0,) if C0 is not None else ()):
         if t.dim() != 3 or not t.is_cuda or t.stride(2) != 1:
