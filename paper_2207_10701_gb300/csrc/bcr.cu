@@ -7,6 +7,7 @@
 #include "bcr.cuh"
 #include "tc_gemm.cuh"
 #include "tc_gemm64.cuh"
+#include "scratch.h"
 
 namespace {
 
@@ -2113,36 +2114,6 @@ __global__ void newton_check_kernel(NewtonFlags f, int n, int batch, int rough, 
 
 constexpr int NEWTON_STEPS = 4;
 
-// Scratch memory in a few regions, handed out in 256-byte units from the region with most left.
-struct Scratch {
-  struct Region {
-    unsigned char* p;
-    size_t bytes, used;
-  };
-  std::vector<Region> r;
-  bool full = false;
-  void add(void* p, int64_t bytes) {
-    if (bytes > 0) r.push_back(Region{(unsigned char*)p, (size_t)bytes, 0});
-  }
-  void reset() {
-    for (Region& g : r) g.used = 0;
-    full = false;
-  }
-  template <typename P> P* take(size_t bytes) {
-    bytes = (bytes + 255) & ~(size_t)255;
-    Region* best = nullptr;
-    for (Region& g : r)
-      if (g.bytes - g.used >= bytes && (!best || g.bytes - g.used > best->bytes - best->used)) best = &g;
-    if (!best) {
-      full = true;
-      return nullptr;
-    }
-    unsigned char* q = best->p + best->used;
-    best->used += bytes;
-    return reinterpret_cast<P*>(q);
-  }
-};
-
 // A split form and its exponents, for up to c operands.
 struct Form {
   unsigned char* f;
@@ -2187,24 +2158,6 @@ struct FwdBuf {
   }
 };
 
-// the most blocks (at most `want`) whose buffers fit, so that the batches are equal; 0: none
-template <typename Place>
-int batch_of(Scratch& w, int want, Place place) {
-  auto fits = [&](int c) {
-    w.reset();
-    place(c);
-    return !w.full;
-  };
-  int lo = 0, hi = std::min(want, 32768);
-  if (want < 1) return 0;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) / 2;
-    if (fits(mid)) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo == 0 ? 0 : (int)ceil_div(want, ceil_div(want, lo));
-}
-
 }  // namespace
 
 // out[z] = D[z]^-1 for z < m (D: stride elements apart, destroyed where the Gauss-Jordan kernel
@@ -2219,6 +2172,7 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
     const int c = std::min(cb, m - k0);
     mem.reset();
     const NewtonBuf w(mem, ny, c);
+    if (mem.full) return cudaErrorInvalidValue;
     float2* a32 = reinterpret_cast<float2*>(w.R);
     float2* x32 = a32 + c * nn;
     double2* R = w.R;
@@ -2359,6 +2313,7 @@ static cudaError_t halves_inverse(float2* D, int64_t stride, float2* out, int n,
     const int c = std::min(cb, m - k0);
     mem.reset();
     const HalvesBuf w(mem, n, c);
+    if (mem.full) return cudaErrorInvalidValue;
     const int h1 = w.h1, h2 = w.h2;
     const int64_t a = (int64_t)h1 * h1, b = (int64_t)h1 * h2, d = (int64_t)h2 * h2;
     float2* A = D + (int64_t)k0 * stride;
@@ -2430,6 +2385,7 @@ static cudaError_t split_level(const double2* D, const double2* L, const double2
     const int p0 = k0 > 0 ? 1 : 0;                 // X, Y of row k0 - 1 come first
     mem.reset();
     const LevelBuf w(mem, ny, c);
+    if (mem.full) return cudaErrorInvalidValue;
     unsigned char *fD = w.D.f, *fO = w.O.f, *fE = w.E.f, *fX = w.X.f, *fY = w.Y.f;
     int32_t *eD = w.D.e, *eO = w.O.e, *eE = w.E.e, *eX = w.X.e, *eY = w.Y.e;
     // L_{2k} for k = k0 .. k0 + c while it exists (index 2k <= n - 1; L_0 is not used)
@@ -2838,6 +2794,7 @@ static cudaError_t split_fwd(BcrHandle* h, Scratch& mem, const double2* Dinv, co
     const int nb1 = p0 + cm;                                            // odd rows from index k0 - p0 on
     mem.reset();
     const FwdBuf w(mem, ny, nq, c);
+    if (mem.full) return cudaErrorInvalidValue;
     unsigned char *fD = w.D.f, *fX = w.X.f, *fY = w.Y.f, *fB = w.B.f;
     int32_t *eD = w.D.e, *eX = w.X.e, *eY = w.Y.e, *eB = w.B.e;
     RCI_CUDA_TRY(launch_sg_split(Dinv + k0 * nn, false, ny, nn, false, ny, ny, 3, cm, fD, eD, nullptr, s));
@@ -2880,6 +2837,7 @@ static cudaError_t split_bwd(BcrHandle* h, Scratch& mem, const double2* X, const
     const int c = std::min(cb, m - k0), cy = std::max(0, std::min(c, my - k0)), nb1 = std::min(c + 1, nk - k0);
     mem.reset();
     const FwdBuf w(mem, ny, nq, c);
+    if (mem.full) return cudaErrorInvalidValue;
     unsigned char *fX = w.X.f, *fY = w.Y.f, *fB = w.B.f;
     int32_t *eX = w.X.e, *eY = w.Y.e, *eB = w.B.e;
     RCI_CUDA_TRY(launch_sg_split(X + k0 * nn, false, ny, nn, false, ny, ny, 3, c, fX, eX, nullptr, s));
@@ -2975,6 +2933,7 @@ static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b
       if (split) {
         mem.reset();
         const FwdBuf w(mem, ny, nq, 1);
+        if (mem.full) return cudaErrorInvalidValue;
         unsigned char *fD = w.D.f, *fB = w.B.f;
         int32_t *eD = w.D.e, *eB = w.B.e;
         RCI_CUDA_TRY(launch_sg_split(Dinv, false, ny, nn, false, ny, ny, 3, 1, fD, eD, nullptr, s));

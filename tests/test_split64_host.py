@@ -21,3 +21,8 @@ def _native(tmp_path, name):
 def test_operand_slots_are_not_overwritten_before_they_are_read(tmp_path):
     r = _native(tmp_path, "slot_ring_check")
     assert r.returncode == 0 and "ring ok" in r.stdout, r.stdout
+
+
+def test_batches_fit_the_scratch_they_are_placed_in(tmp_path):
+    r = _native(tmp_path, "scratch_check")
+    assert r.returncode == 0 and "scratch ok" in r.stdout, r.stdout
