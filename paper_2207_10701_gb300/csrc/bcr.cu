@@ -2047,6 +2047,9 @@ cudaError_t bcr_read_status(BcrHandle* h, int32_t* st, cudaStream_t s, double* g
   return cudaSuccess;
 }
 
+cudaError_t bcr_clear_timeout(BcrHandle* h, cudaStream_t s) {
+  return cudaMemsetAsync(h->status, 0, sizeof(int32_t), s);
+}
 
 // ===================================================================== FP64 on the tensor cores
 // The FP64 factorisation runs its block products through the digit split of tc_gemm64.cu and its

@@ -41,6 +41,8 @@ cudaError_t bcr_solve(BcrHandle* h, const double2* cx, const void* b, void* x, i
 // growth, also the growth estimate of the last factorisation: the largest |re|, |im| of the
 // blocks it inverted (the Schur complements of every level) over that of A's coefficients.
 cudaError_t bcr_read_status(BcrHandle* h, int32_t* st, cudaStream_t s, double* growth = nullptr);
+// The status word after a reported expired wait: the next solve starts anew.
+cudaError_t bcr_clear_timeout(BcrHandle* h, cudaStream_t s);
 int bcr_precision(const BcrHandle* h);
 // Arithmetic of an FP32 handle from its next bcr_factor on: false (the default) runs the block
 // inversions and the products of the factorisation and of the several-right-hand-side solve

@@ -387,6 +387,17 @@ rci_status residual_ratio(rci_grid* g, const double2* b, const double2* x, doubl
   return RCI_OK;
 }
 
+// Solves with several right-hand sides run tensor-core products with bounded waits: RCI_ETIMEOUT where
+// one on h's factorisation has expired, else the status that the solve came to.
+rci_status checked_solve(rci_grid* g, BcrHandle* h, int nrhs, rci_status st) {
+  if (nrhs == 1 || (st != RCI_OK && st != RCI_ENUMERIC)) return st;
+  int32_t dst = 0;
+  CK(bcr_read_status(h, &dst, g->s), "solve status");
+  if (dst != DEV_TIMEOUT) return st;
+  CK(bcr_clear_timeout(h, g->s), "solve status");  // (the factors are as they were)
+  return fail(g, RCI_ETIMEOUT, "a bounded tensor-core wait expired");
+}
+
 // FP64 refinement on an FP64 factorisation h: x = A^-1 b, then corrections d while the
 // FP64 stencil residual is above tol64 (at most max_refine64 steps).
 rci_status solve64(rci_grid* g, BcrHandle* h, const double2* b, double2* x, double2* r, double2* d,
@@ -673,7 +684,7 @@ rci_status refined_solve(rci_grid* g, const double2* b, double2* x, double2* r, 
   bool fell_back = false;
   rci_status st = RCI_OK;
   if (g->d.prec == RCI_FP64) {
-    st = solve64(g, g->bcr, b, x, r, (double2*)a32, nrhs, &it, &worst);
+    st = checked_solve(g, g->bcr, nrhs, solve64(g, g->bcr, b, x, r, (double2*)a32, nrhs, &it, &worst));
     if (st != RCI_OK) return st;
   } else {
     bool need64 = g->use64;
@@ -697,7 +708,7 @@ rci_status refined_solve(rci_grid* g, const double2* b, double2* x, double2* r, 
       st = ensure_corr64(g, n);
       if (st != RCI_OK) return st;
       it = 0;
-      st = solve64(g, g->bcr64, b, x, r, g->corr64, nrhs, &it, &worst);
+      st = checked_solve(g, g->bcr64, nrhs, solve64(g, g->bcr64, b, x, r, g->corr64, nrhs, &it, &worst));
       if (st != RCI_OK) return st;
       fell_back = true;
     }
@@ -710,10 +721,9 @@ rci_status refined_solve(rci_grid* g, const double2* b, double2* x, double2* r, 
     info->krylov_steps = kry;
     info->simt_refactor = bcr_simt(g->bcr) ? 1 : 0;
   }
-  if (nrhs > 1) {  // the multi-RHS solve runs tensor-core GEMMs with bounded waits
-    int32_t dst = 0;
-    CK(bcr_read_status(g->bcr, &dst, g->s), "solve status");
-    if (dst == DEV_TIMEOUT) return fail(g, RCI_ETIMEOUT, "a bounded tensor-core wait expired");
+  if (g->d.prec != RCI_FP64) {
+    st = checked_solve(g, g->bcr, nrhs, RCI_OK);
+    if (st != RCI_OK) return st;
   }
   double tol = (g->d.prec == RCI_FP64 || fell_back) ? 1e-9 : g->tol32;
   if (worst > tol) return fail(g, RCI_ENOCONV, "iterative refinement did not converge");
