@@ -60,7 +60,7 @@ cudaError_t launch_planewave_row(const GridGeom& g, double theta_out, double2* c
 cudaError_t launch_virtual_focus_row(const GridGeom& g, double x_f, int d_rows, double2* crow,
                                      double* scratch /* >= 2*VF_ORDER + 6*VF_NODES doubles */,
                                      bool have_rule /* scratch holds the rule of an earlier call */,
-                                     double2* part /* >= ny * n_src */, cudaStream_t s);
+                                     double2* part /* nx * ny */, cudaStream_t s);
 constexpr int VF_PANELS = 256, VF_ORDER = 32, VF_NODES = VF_PANELS * VF_ORDER;
 // scatter a row vector into a zeroed full-grid vector: b[(npml+t)*ny + row] = crow[t] (conj if asked)
 cudaError_t launch_scatter_row(const GridGeom& g, const double2* crow, int row, double2* b,

@@ -8,6 +8,8 @@
 // * Gauss-Legendre rules (Sec. 5.2) and W(m h) in closed form (Eq. 4 and the
 //   annulus formula of Sec. 5.1, with the cos(theta) Jacobian of the unit-power
 //   amplitude: W(D) = int rho cos(theta) exp(i k_s sin(theta) D) dtheta).
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace {
@@ -184,11 +186,13 @@ __global__ void vf_tables_kernel(GridGeom g, int D, const double* __restrict__ g
 // anchor at x_c between two columns and a column at x_c +- d, d = (j + 1/2) h,
 //   cos(k (x_f - x_c -+ d)) = cos(k (x_f - x_c)) cos(k d) +- sin(k (x_f - x_c)) sin(k d),
 // and the sums over the nodes of f cos cos and f sin sin serve the columns on both sides.  An
-// anchor serves 64 columns, a block VF_GROUP anchors and a chunk of the nodes: per node it
+// anchor serves 64 columns, a block up to VF_GROUP anchors and a chunk of the nodes: per node it
 // evaluates 2 sincos for each anchor and 2 for each of the 32 distances instead of 2 cosines for
 // each column, and 3 FMAs per node and column remain.  The rounding of k (x_f - x_c) is that of
 // the direct form's argument.  Bound by the FP64 pipe: 2.67 -> 0.28 ms at 4000 columns (one cosine
-// per node and column: 65.5 million of them).  The chunks' sums are added in a fixed order.
+// per node and column: 65.5 million of them), the row whole.  Anchors beyond the last column take no
+// part: 64 columns of 64 rows 0.35 -> 0.13 ms (0.21 with a cosine per node and column).  The chunks'
+// sums are added in a fixed order.
 constexpr int VF_SIDE = 32;            // columns on either side of an anchor
 constexpr int VF_WARPS = 8, VF_PER_WARP = 4, VF_GROUP = VF_WARPS * VF_PER_WARP;
 constexpr int VF_TILE = 16;            // nodes staged at a time
@@ -201,8 +205,12 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
   __shared__ double pc[VF_GROUP][VF_TILE][6];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int a0 = blockIdx.x * VF_GROUP;
+  // the block's anchors up to the last column (warp w takes w, w + VF_WARPS, ..: `mine` of them)
+  const int anchors = min(VF_GROUP, (g.n_src + 2 * VF_SIDE - 1) / (2 * VF_SIDE) - a0);
+  const int mine = (anchors - warp + VF_WARPS - 1) / VF_WARPS;
+  const int end = min((int)(blockIdx.y + 1) * nodes, VF_NODES);
   double er[VF_PER_WARP] = {}, ei[VF_PER_WARP] = {}, orr[VF_PER_WARP] = {}, oi[VF_PER_WARP] = {};
-  for (int n0 = blockIdx.y * nodes; n0 < (int)(blockIdx.y + 1) * nodes; n0 += VF_TILE) {
+  for (int n0 = blockIdx.y * nodes; n0 < end; n0 += VF_TILE) {
     // evanescent nodes that have decayed below VF_NONE on the way count for nothing beside the
     // propagating ones (weights of some 1e-3): 60 % of them at 100 rows, 85 % at 400
     const bool ev = __syncthreads_or(threadIdx.x < VF_TILE &&
@@ -217,7 +225,7 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
       sincos(tab[4 * VF_NODES + 2 * n] * d, &v.y, &v.x);
       qe[e / VF_SIDE][j] = v;
     }
-    for (int e = threadIdx.x; e < VF_GROUP * VF_TILE; e += 32 * VF_WARPS) {
+    for (int e = threadIdx.x; e < anchors * VF_TILE; e += 32 * VF_WARPS) {
       const int n = n0 + e % VF_TILE, a = e / VF_TILE;
       const double delta = x_f - (double)(2 * VF_SIDE * (a0 + a) + VF_SIDE) * g.h;
       double s, c;
@@ -240,7 +248,8 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
       const double2 u = qp[n][lane];
 #pragma unroll
       for (int i = 0; i < VF_PER_WARP; ++i) {
-        const double* o = pc[warp * VF_PER_WARP + i][n];
+        if (i >= mine) break;
+        const double* o = pc[i * VF_WARPS + warp][n];
         er[i] = fma(o[0], u.x, er[i]);
         ei[i] = fma(o[1], u.x, ei[i]);
         orr[i] = fma(o[2], u.y, orr[i]);
@@ -253,7 +262,8 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
       const double2 v = qe[n][lane];
 #pragma unroll
       for (int i = 0; i < VF_PER_WARP; ++i) {
-        const double* o = pc[warp * VF_PER_WARP + i][n];
+        if (i >= mine) break;
+        const double* o = pc[i * VF_WARPS + warp][n];
         er[i] = fma(o[4], v.x, er[i]);
         orr[i] = fma(o[5], v.y, orr[i]);
       }
@@ -262,7 +272,8 @@ vf_sums_kernel(GridGeom g, double x_f, const double* __restrict__ tab, int nodes
   double2* out = part + (int64_t)blockIdx.y * g.n_src;
 #pragma unroll
   for (int i = 0; i < VF_PER_WARP; ++i) {
-    const int c = 2 * VF_SIDE * (a0 + warp * VF_PER_WARP + i) + VF_SIDE;  // first column to the right
+    if (i >= mine) break;
+    const int c = 2 * VF_SIDE * (a0 + i * VF_WARPS + warp) + VF_SIDE;  // first column to the right
     if (c + lane < g.n_src) out[c + lane] = mkc(er[i] + orr[i], ei[i] + oi[i]);
     if (c - 1 - lane < g.n_src) out[c - 1 - lane] = mkc(er[i] - orr[i], ei[i] - oi[i]);
   }
@@ -422,11 +433,22 @@ cudaError_t launch_virtual_focus_row(const GridGeom& g, double x_f, int d_rows, 
   if (!have_rule) RCI_CUDA_TRY(launch_gauss_legendre(VF_ORDER, -1.0, 1.0, gx, gw, s));
   vf_tables_kernel<<<(unsigned)ceil_div(VF_NODES, 128), 128, 0, s>>>(g, d_rows, gx, gw, tab); rci_note_launch();
   RCI_CUDA_TRY(cudaGetLastError());
-  // 128 chunks of 64 nodes where the scratch holds as many partial rows (ny >= 128), else fewer
-  int chunks = 128;
-  while (chunks > g.ny) chunks >>= 1;
-  const unsigned groups = (unsigned)ceil_div(g.n_src, 2 * VF_SIDE * VF_GROUP);
-  vf_sums_kernel<<<dim3(groups, (unsigned)chunks), 32 * VF_WARPS, 0, s>>>(g, x_f, tab, VF_NODES / chunks, part);
+  // Chunks of four tiles of nodes; where the scratch (nx ny) does not hold as many partial rows
+  // (ny < 128), more tiles, so that the busiest SM has least to do: a second block on an SM costs about
+  // five sixths of the time it takes alone (4000 columns: 128 blocks of 8 tiles 0.36 ms, 172 of 6 0.42,
+  // 148 of 7 0.31, 256 of 4 0.30).
+  const int groups = (int)ceil_div(g.n_src, 2 * VF_SIDE * VF_GROUP);
+  const int tiles = VF_NODES / VF_TILE, least = (int)ceil_div(tiles, (int64_t)g.nx * g.ny / g.n_src);
+  int per = std::max(4, least), best = 0;
+  for (int t = least; least > 4 && (best == 0 || t <= 16); ++t) {
+    const int blocks = (int)ceil_div(groups * ceil_div(tiles, t), 152), cost = (blocks == 1 ? 6 : 5 * blocks) * t;
+    if (best == 0 || cost < best) {
+      per = t;
+      best = cost;
+    }
+  }
+  const int nodes = per * VF_TILE, chunks = (int)ceil_div(tiles, per);
+  vf_sums_kernel<<<dim3((unsigned)groups, (unsigned)chunks), 32 * VF_WARPS, 0, s>>>(g, x_f, tab, nodes, part);
   rci_note_launch();
   RCI_CUDA_TRY(cudaGetLastError());
   vf_join_kernel<<<(unsigned)ceil_div(g.n_src, 128), 128, 0, s>>>(g, part, chunks, crow);
