@@ -3152,8 +3152,10 @@ static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, 
     // Many FP64 rows: one thread per row.  The FP64 pipe takes as long for a warp's one busy lane as for
     // all of them, so with a warp per row 2020 rows of 160 take 340 us a sweep; with a thread per row
     // 235 and 255.  Few rows are bound by one row's chain of operations, which is shorter on a warp's
-    // staged copies (220 rows of 128: 84 us against 170 and 200).
-    const bool thread_per_row = sizeof(T) == 8 && m0 > 1024;
+    // staged copies (220 rows of 128: 84 us against 170 and 200).  The line lies where a ninth warp comes
+    // to an SM: whole solves of 64 to 224 rows take 3 to 4 % less with warps at 1200 columns, 2 to 4 % less
+    // with threads at 1400.
+    const bool thread_per_row = sizeof(T) == 8 && m0 > 8 * 152;
     if (m0 > 0) {
       if (thread_per_row) {
         fwd0_kernel<T><<<(unsigned)ceil_div(m0, 32), 32, 0, s>>>(
