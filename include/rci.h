@@ -440,11 +440,14 @@ uint64_t rci_kernel_launches(void);
  * solve rests on it):  out[z] = src[z]^{-1},  z < batch.
  * src, out: DEVICE arrays of batch row-major n x n blocks, contiguous, interleaved complex --
  * complex64 for prec = RCI_FP32_REFINE, complex128 for RCI_FP64; must not overlap; src may
- * be overwritten for n > 160.  kernel: 0 the factorisation's choice, 1 the SIMT Gauss-Jordan
- * kernels, 2 the tensor-core Gauss-Jordan (FP32 and n <= 160 only: tcgen05 3xTF32 panel
- * updates on the block held in tensor memory).  Pivot: largest |re| + |im| among the rows
- * not yet used.  Synchronises `stream` (cudaStream_t or NULL) and allocates a 4-byte
- * status word.  Errors: EINVAL, ESINGULAR (a zero pivot; out is then undefined), ETIMEOUT. */
+ * be overwritten for n > 160 and kernel 3.  kernel: 0 the Gauss-Jordan kernel for the size, 1 the
+ * SIMT Gauss-Jordan kernels, 2 the tensor-core Gauss-Jordan (FP32 and n <= 160 only: tcgen05
+ * 3xTF32 panel updates on the block held in tensor memory), 3 the factorisation's Newton forms
+ * (FP64, n <= 248: digit-split products on an FP32 inverse; FP32, even 160 < n <= 248: inversion
+ * by halves and one step), whose blocks that do not contract go to kernel 1; allocates their
+ * scratch.  Pivot: largest |re| + |im| among the rows not yet used.  Synchronises `stream`
+ * (cudaStream_t or NULL) and allocates a 4-byte status word.  Errors: EINVAL, ENOMEM, ESINGULAR (a
+ * zero pivot; out is then undefined), ETIMEOUT. */
 rci_status rci_block_inverse(const void* src, void* out, int64_t n, int64_t batch, int32_t prec,
                              int32_t kernel, void* stream);
 
@@ -457,14 +460,15 @@ rci_status rci_block_inverse(const void* src, void* out, int64_t n, int64_t batc
  * RCI_FP32_REFINE) or complex128 (RCI_FP64), leading dimensions lda, ldb, ldc0, ldc and element
  * strides sA, sB, sC0, sC between batch members (in complex elements); C0 may be NULL
  * (beta ignored).  C may equal C0 (same element positions), no other overlap.
- * kernel: 0 = the factorisation's dispatch; 1 = tensor cores (3xTF32 tcgen05), operands
- * staged through registers into shared memory; 2 = tensor cores fed by TMA with the A
- * operand in tensor memory (needs 2 <= N <= 160 and even, 16-byte aligned A, B, C, C0, even
- * leading dimensions and, for batch > 1, even positive sA, sB); 3 = SIMT; 4 = the digit split
- * of FP64 on the tensor cores (FP64 only, K <= 248, alpha = 1 or -1, beta = 1 with a C0; allocates
- * its operands' split forms).  Kernels 1 and 2 are FP32 only; the SIMT kernel (3, and 0 where it dispatches there: FP64, or batches too
- * small to fill the GPU) has no form with both operands transposed.  Synchronises `stream` (cudaStream_t or NULL) and allocates a 4-byte status
- * word.  Errors: EINVAL (sizes, a kernel that does not apply), ETIMEOUT, ECUDA. */
+ * kernel: 0 = the dispatch by size (FP64: SIMT; the factorisation's levels take 4); 1 = tensor
+ * cores (3xTF32 tcgen05), operands staged through registers into shared memory; 2 = tensor cores
+ * fed by TMA with the A operand in tensor memory (needs 2 <= N <= 160 and even, 16-byte aligned
+ * A, B, C, C0, even leading dimensions and, for batch > 1, even positive sA, sB); 3 = SIMT; 4 = the
+ * digit split of FP64 on the tensor cores (FP64 only, K <= 248, alpha = 1 or -1, beta = 1 with a
+ * C0; allocates its operands' split forms).  Kernels 1 and 2 are FP32 only; the SIMT kernel (3, and
+ * 0 where it dispatches there: FP64, or batches too small to fill the GPU) has no form with both
+ * operands transposed.  Synchronises `stream` (cudaStream_t or NULL) and allocates a 4-byte status
+ * word.  Errors: EINVAL (sizes, a kernel that does not apply), ENOMEM, ETIMEOUT, ECUDA. */
 rci_status rci_cgemm_batched(int64_t M, int64_t N, int64_t K, int32_t ta, int32_t tb,
                              double alpha, const void* A, int64_t lda, int64_t sA, const void* B,
                              int64_t ldb, int64_t sB, double beta, const void* C0, int64_t ldc0,

@@ -3245,6 +3245,23 @@ cudaError_t bcr_solve(BcrHandle* h, const double2* cx, const void* b, void* x, i
 cudaError_t bcr_block_inverse(const void* src, void* out, int n, int batch, int prec, int kernel,
                               int32_t* status, cudaStream_t s) {
   const int64_t nn = (int64_t)n * n;
+  if (kernel == 3) {
+    const bool f64 = prec == RCI_FP64;
+    if (n > SG_KMAX || (!f64 && (n <= 160 || n % 2))) return cudaErrorInvalidValue;
+    Scratch need, mem;
+    need.add(nullptr, (int64_t)1 << 60);  // (only counted)
+    if (f64) NewtonBuf(need, n, batch);
+    else HalvesBuf(need, n, batch);
+    void* w = nullptr;
+    RCI_CUDA_TRY(cudaMalloc(&w, need.r[0].used));
+    mem.add(w, (int64_t)need.r[0].used);
+    cudaError_t e = f64 ? split_inverse((double2*)src, nn, (double2*)out, n, batch, mem, status, s)
+                        : halves_inverse((float2*)src, nn, (float2*)out, n, batch, mem, status, s);
+    if (e == cudaErrorNotSupported) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(w);
+    return e;
+  }
   if (prec == RCI_FP64) {
     if (kernel == 2) return cudaErrorInvalidValue;
     return launch_gj<double>((double2*)src, nn, (double2*)out, nn, n, batch, status, s);

@@ -1501,7 +1501,7 @@ uint64_t rci_kernel_launches(void) { return g_launches.load(std::memory_order_re
 rci_status rci_block_inverse(const void* src, void* out, int64_t n, int64_t batch, int32_t prec,
                              int32_t kernel, void* stream) {
   if (!src || !out || n < 1 || n > 1024 || batch < 1 || batch > (1 << 24) || kernel < 0 ||
-      kernel > 2 || (prec != RCI_FP64 && prec != RCI_FP32_REFINE))
+      kernel > 3 || (prec != RCI_FP64 && prec != RCI_FP32_REFINE))
     return RCI_EINVAL;
   if (kernel == 2 && (prec != RCI_FP32_REFINE || n > 160)) return RCI_EINVAL;
   cudaStream_t s = (cudaStream_t)stream;

@@ -447,7 +447,8 @@ def measure_peaks(device: int = 0) -> dict:
 def block_inverse(blocks, kernel: int = 0, stream=None):
     """Inverses of a batch of complex blocks (CUDA tensor [batch, n, n], complex64 or
     complex128) with the factorisation's block-inverse kernels (rci_block_inverse);
-    kernel 0 = its choice, 1 = SIMT, 2 = tensor cores (complex64, n <= 160)."""
+    kernel 0 = Gauss-Jordan by size, 1 = SIMT, 2 = tensor cores (complex64, n <= 160), 3 = Newton
+    steps (complex128, n <= 248; complex64, even n from 162 to 248)."""
     torch = _torch()
     if blocks.dim() != 3 or blocks.shape[1] != blocks.shape[2] or not blocks.is_cuda:
         raise ValueError("blocks: CUDA tensor [batch, n, n]")
