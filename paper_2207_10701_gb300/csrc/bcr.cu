@@ -2121,7 +2121,7 @@ cudaError_t bcr_clear_timeout(BcrHandle* h, cudaStream_t s) {
 // block inverses as Newton iterations on an FP32 inverse, X <- X + X (I - D X), with those products:
 // the FP64 pipe does neither.  At ny = 160 a product takes 1.2 us of the whole GPU where the FP64
 // GEMM took 28, and an inverse of one block alone 0.4 ms where the FP64 Gauss-Jordan took 4.9: a
-// new design of 500 cells 404 -> 38 ms, of 50 cells (ny = 128) 54 -> 5.4 ms.
+// new design of 500 cells 404 -> 39 ms, of 50 cells (ny = 128) 54 -> 5.5 ms.
 // A block whose iteration does not contract (an FP32 inverse that resolves nothing, entries outside
 // the FP32 range, a singular block) goes to the FP64 Gauss-Jordan kernel, which also reports zero
 // pivots, so the factorisation accepts and refuses what it did.
@@ -2314,7 +2314,8 @@ static cudaError_t split_inverse(double2* D, int64_t stride, double2* out, int n
 //   2. pivoting only within the halves costs digits, so one Newton step X + X (I - A X) follows with
 //      the residual formed through the digit split (SG_SMALL: error 2^-28, where FP32 rounds at 2^-24): the
 //      inverse it leaves is closer to the exact one than the SIMT kernel's.
-// Blocks whose step would leave more than that kernel does (residual entries of some 1e-5 at n = 224),
+// Blocks whose step would leave more than that kernel does (n m^2 > 2e-6 for residual entries of m: from
+// 9.4e-5 on at n = 224, where ordinary blocks leave some 1e-5),
 // or whose halves are singular, go to the SIMT kernel, which also reports zero pivots.
 namespace {
 
@@ -2574,7 +2575,6 @@ static cudaError_t factor_t(BcrHandle* h, const double2* dg, const double2* cx, 
   const cplx<T> one = mkc(T(1), T(0)), mone = mkc(T(-1), T(0)), zero = czero<T>();
   int cur = 0;
   auto store = (cplx<T>*)h->store;
-  // FP64 on the tensor cores where the scratch holds at least one block
   // the scratch of an inversion (sch == false) or of the products of level l
   auto scratch_of = [&](int l, bool sch) {
     Scratch w;
@@ -3073,12 +3073,11 @@ static cudaError_t solve_multi(BcrHandle* h, const double2* cx, const cplx<T>* b
 
 template <typename T>
 static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, cplx<T>* x, cudaStream_t s) {
-  constexpr int nrhs = 1;
   const int nx = h->nx, ny = h->ny;
   const int64_t nn = (int64_t)ny * ny;
-  const int64_t row = (int64_t)ny * nrhs;
+  const int64_t row = ny;
   const int m0 = (int)h->m[0], n1 = (nx + 1) / 2;
-  RCI_CUDA_TRY(bcr_reserve_ws(h, nrhs));
+  RCI_CUDA_TRY(bcr_reserve_ws(h, 1));
   // carve the workspace
   cplx<T>* p = (cplx<T>*)h->ws;
   cplx<T>* t0 = p;
@@ -3118,11 +3117,11 @@ static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, 
   const int dense = h->Lf - 1, l0 = m0 > 0 ? 1 : 0;
   ProfScope ps(h->prof, PF_SOLVE, s, sflops, sbytes, l0 + 1 + dense + 1 + dense + 1);
 
-    if (ny % vec16<T>::per != 0 || ny > 256 * vec16<T>::per)
-      return cudaErrorInvalidValue;  // (grid creation keeps ny within these limits)
-    const int smax = (int)ceil_div(ny, 32 * vec16<T>::per);
-    const unsigned nch = (unsigned)ceil_div(ny, RC);
-    const size_t red_smem = (size_t)2 * CH_WARPS * RC * sizeof(cplx<T>);
+  if (ny % vec16<T>::per != 0 || ny > 256 * vec16<T>::per)
+    return cudaErrorInvalidValue;  // (grid creation keeps ny within these limits)
+  const int smax = (int)ceil_div(ny, 32 * vec16<T>::per);
+  const unsigned nch = (unsigned)ceil_div(ny, RC);
+  const size_t red_smem = (size_t)2 * CH_WARPS * RC * sizeof(cplx<T>);
 #define RCI_SMAX_DISPATCH(KERNEL, GRID, SMEM, ...)                                   \
   do {                                                                               \
     switch (smax) {                                                                  \
@@ -3138,96 +3137,96 @@ static cudaError_t solve_one(BcrHandle* h, const double2* cx, const cplx<T>* b, 
     rci_note_launch();                                                               \
     RCI_CUDA_TRY(cudaGetLastError());                                                \
   } while (0)
-    // the chunked level-0 backward pass reads b while other blocks write x: no aliasing
-    const cplx<T>* bsrc = b;
-    if ((const void*)b == (const void*)x) return cudaErrorInvalidValue;
-    // ---- level 0 forward: t0[k] = T_{2k+1}^{-1} b[2k+1] by tridiagonal sweeps
-    const size_t trs_smem = TRS_WARPS * trs_smem_per_warp<T>(ny);
-    auto trs_attr = [&](auto kern) -> cudaError_t {
-      return trs_smem > 48 * 1024 ? cudaFuncSetAttribute(kern,
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)trs_smem)
-                                  : cudaSuccess;
-    };
-    // Many FP64 rows: one thread per row.  The FP64 pipe takes as long for a warp's one busy lane as for
-    // all of them, so with a warp per row 2020 rows of 160 take 340 us a sweep; with a thread per row
-    // 235 and 255.  Few rows are bound by one row's chain of operations, which is shorter on a warp's
-    // staged copies (220 rows of 128: 84 us against 170 and 200).  The line lies where a ninth warp comes
-    // to an SM: whole solves of 64 to 224 rows take 3 to 4 % less with warps at 1200 columns, 2 to 4 % less
-    // with threads at 1400.
-    const bool thread_per_row = sizeof(T) == 8 && m0 > 8 * 152;
-    if (m0 > 0) {
-      if (thread_per_row) {
-        fwd0_kernel<T><<<(unsigned)ceil_div(m0, 32), 32, 0, s>>>(
-            bsrc, t0, ny, m0, 1, 1, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
-            (const cplx<T>*)h->tdu2, h->tpiv);
-      } else {
-        RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, false>));
-        tri_rows_solve_kernel<T, false><<<(unsigned)ceil_div(m0, TRS_WARPS), 32 * TRS_WARPS, trs_smem, s>>>(
-            (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
-            (const cplx<T>*)h->tdu2, h->tpiv, bsrc, nullptr, cx, t0, nx, ny, m0);
-      }
-      rci_note_launch();
-      RCI_CUDA_TRY(cudaGetLastError());
-    }
-    {
-      int64_t nt = (int64_t)n1 * row;
-      keep0_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(bsrc, t0, cx, B[1], nx, ny, n1, 1, 1);
-      rci_note_launch();
-      RCI_CUDA_TRY(cudaGetLastError());
-    }
-    // ---- dense levels forward: level 1 from the kept rows of level 0; every later level forms
-    // its rows from the level before (the kept-row update fused into its forward kernel), the
-    // P and Q of odd levels in (P, Q), of even levels in (P2, Q2)
-    auto Pl = [&](int l) { return (l & 1) ? P : P2; };
-    auto Ql = [&](int l) { return (l & 1) ? Q : Q2; };
-    for (int l = 1; l < h->Lf; ++l) {
-      const int n = (int)h->n[l], m = (int)h->m[l];
-      const cplx<T>* Dinv = store + h->off[l];
-      const cplx<T>* X = Dinv + (int64_t)m * nn;
-      const cplx<T>* Y = X + (int64_t)m * nn;
-      if (l == 1) {
-        RCI_SMAX_DISPATCH(fwd_chunk_kernel, dim3(m, nch), ny * sizeof(cplx<T>) + red_smem, Dinv,
-                          X, Y, B[1], tl[1], Pl(1), Ql(1), n, ny);
-      } else {
-        RCI_SMAX_DISPATCH(fwd_keep_chunk_kernel, dim3((unsigned)h->n[l + 1], nch),
-                          ny * sizeof(cplx<T>) + red_smem, Dinv, X, Y, B[l - 1], Pl(l - 1),
-                          Ql(l - 1), (int)h->m[l - 1], B[l], tl[l], Pl(l), Ql(l), n, ny);
-      }
-    }
-    // ---- single remaining row (from the level before it when there is one, written straight
-    // to B[Lf], which nothing reads as input then)
-    if (h->Lf >= 2) {
-      const int lp = h->Lf - 1;
-      RCI_SMAX_DISPATCH(mv_keep_chunk_kernel, dim3(1, nch), ny * sizeof(cplx<T>),
-                        store + h->final_off, B[lp], Pl(lp), Ql(lp), (int)h->m[lp], B[h->Lf], ny);
-    } else {
-      RCI_SMAX_DISPATCH(mv_chunk_kernel, dim3(1, nch), ny * sizeof(cplx<T>), store + h->final_off,
-                        B[h->Lf], (int64_t)0, (int64_t)0, xf, ny);
-      RCI_CUDA_TRY(cudaMemcpyAsync(B[h->Lf], xf, row * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
-    }
-    // ---- dense levels backward (the solution of level l overwrites B[l])
-    for (int l = h->Lf - 1; l >= 1; --l) {
-      const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
-      const cplx<T>* Dinv = store + h->off[l];
-      const cplx<T>* X = Dinv + (int64_t)m * nn;
-      const cplx<T>* Y = X + (int64_t)m * nn;
-      RCI_SMAX_DISPATCH(bwd_chunk_kernel, dim3(nk, nch), 3 * ny * sizeof(cplx<T>), X, Y, tl[l],
-                        B[l + 1], B[l], n, m, ny);
-    }
-    // ---- level 0 backward by tridiagonal sweeps (and the kept rows copied)
+  // the chunked level-0 backward pass reads b while other blocks write x: no aliasing
+  const cplx<T>* bsrc = b;
+  if ((const void*)b == (const void*)x) return cudaErrorInvalidValue;
+  // ---- level 0 forward: t0[k] = T_{2k+1}^{-1} b[2k+1] by tridiagonal sweeps
+  const size_t trs_smem = TRS_WARPS * trs_smem_per_warp<T>(ny);
+  auto trs_attr = [&](auto kern) -> cudaError_t {
+    return trs_smem > 48 * 1024 ? cudaFuncSetAttribute(kern,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)trs_smem)
+                                : cudaSuccess;
+  };
+  // Many FP64 rows: one thread per row.  The FP64 pipe takes as long for a warp's one busy lane as for
+  // all of them, so with a warp per row 2020 rows of 160 take 340 us a sweep; with a thread per row
+  // 235 and 255.  Few rows are bound by one row's chain of operations, which is shorter on a warp's
+  // staged copies (220 rows of 128: 84 us against 170 and 200).  The line lies where a ninth warp comes
+  // to an SM: whole solves of 64 to 224 rows take 3 to 4 % less with warps at 1200 columns, 2 to 4 % less
+  // with threads at 1400.
+  const bool thread_per_row = sizeof(T) == 8 && m0 > 8 * 152;
+  if (m0 > 0) {
     if (thread_per_row) {
-      bwd0_kernel<T><<<(unsigned)ceil_div(n1, 32), 32, 0, s>>>(
-          bsrc, B[1], cx, x, nx, ny, n1, 1, 1, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv,
-          (const cplx<T>*)h->tdu, (const cplx<T>*)h->tdu2, h->tpiv);
+      fwd0_kernel<T><<<(unsigned)ceil_div(m0, 32), 32, 0, s>>>(
+          bsrc, t0, ny, m0, 1, 1, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+          (const cplx<T>*)h->tdu2, h->tpiv);
     } else {
-      RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, true>));
-      tri_rows_solve_kernel<T, true><<<(unsigned)ceil_div(n1, TRS_WARPS), 32 * TRS_WARPS, trs_smem, s>>>(
+      RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, false>));
+      tri_rows_solve_kernel<T, false><<<(unsigned)ceil_div(m0, TRS_WARPS), 32 * TRS_WARPS, trs_smem, s>>>(
           (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
-          (const cplx<T>*)h->tdu2, h->tpiv, bsrc, B[1], cx, x, nx, ny, n1);
+          (const cplx<T>*)h->tdu2, h->tpiv, bsrc, nullptr, cx, t0, nx, ny, m0);
     }
     rci_note_launch();
     RCI_CUDA_TRY(cudaGetLastError());
+  }
+  {
+    int64_t nt = (int64_t)n1 * row;
+    keep0_kernel<T><<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(bsrc, t0, cx, B[1], nx, ny, n1, 1, 1);
+    rci_note_launch();
+    RCI_CUDA_TRY(cudaGetLastError());
+  }
+  // ---- dense levels forward: level 1 from the kept rows of level 0; every later level forms
+  // its rows from the level before (the kept-row update fused into its forward kernel), the
+  // P and Q of odd levels in (P, Q), of even levels in (P2, Q2)
+  auto Pl = [&](int l) { return (l & 1) ? P : P2; };
+  auto Ql = [&](int l) { return (l & 1) ? Q : Q2; };
+  for (int l = 1; l < h->Lf; ++l) {
+    const int n = (int)h->n[l], m = (int)h->m[l];
+    const cplx<T>* Dinv = store + h->off[l];
+    const cplx<T>* X = Dinv + (int64_t)m * nn;
+    const cplx<T>* Y = X + (int64_t)m * nn;
+    if (l == 1) {
+      RCI_SMAX_DISPATCH(fwd_chunk_kernel, dim3(m, nch), ny * sizeof(cplx<T>) + red_smem, Dinv,
+                        X, Y, B[1], tl[1], Pl(1), Ql(1), n, ny);
+    } else {
+      RCI_SMAX_DISPATCH(fwd_keep_chunk_kernel, dim3((unsigned)h->n[l + 1], nch),
+                        ny * sizeof(cplx<T>) + red_smem, Dinv, X, Y, B[l - 1], Pl(l - 1),
+                        Ql(l - 1), (int)h->m[l - 1], B[l], tl[l], Pl(l), Ql(l), n, ny);
+    }
+  }
+  // ---- single remaining row (from the level before it when there is one, written straight
+  // to B[Lf], which nothing reads as input then)
+  if (h->Lf >= 2) {
+    const int lp = h->Lf - 1;
+    RCI_SMAX_DISPATCH(mv_keep_chunk_kernel, dim3(1, nch), ny * sizeof(cplx<T>),
+                      store + h->final_off, B[lp], Pl(lp), Ql(lp), (int)h->m[lp], B[h->Lf], ny);
+  } else {
+    RCI_SMAX_DISPATCH(mv_chunk_kernel, dim3(1, nch), ny * sizeof(cplx<T>), store + h->final_off,
+                      B[h->Lf], (int64_t)0, (int64_t)0, xf, ny);
+    RCI_CUDA_TRY(cudaMemcpyAsync(B[h->Lf], xf, row * sizeof(cplx<T>), cudaMemcpyDeviceToDevice, s));
+  }
+  // ---- dense levels backward (the solution of level l overwrites B[l])
+  for (int l = h->Lf - 1; l >= 1; --l) {
+    const int n = (int)h->n[l], m = (int)h->m[l], nk = (int)h->n[l + 1];
+    const cplx<T>* Dinv = store + h->off[l];
+    const cplx<T>* X = Dinv + (int64_t)m * nn;
+    const cplx<T>* Y = X + (int64_t)m * nn;
+    RCI_SMAX_DISPATCH(bwd_chunk_kernel, dim3(nk, nch), 3 * ny * sizeof(cplx<T>), X, Y, tl[l],
+                      B[l + 1], B[l], n, m, ny);
+  }
+  // ---- level 0 backward by tridiagonal sweeps (and the kept rows copied)
+  if (thread_per_row) {
+    bwd0_kernel<T><<<(unsigned)ceil_div(n1, 32), 32, 0, s>>>(
+        bsrc, B[1], cx, x, nx, ny, n1, 1, 1, (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv,
+        (const cplx<T>*)h->tdu, (const cplx<T>*)h->tdu2, h->tpiv);
+  } else {
+    RCI_CUDA_TRY(trs_attr(tri_rows_solve_kernel<T, true>));
+    tri_rows_solve_kernel<T, true><<<(unsigned)ceil_div(n1, TRS_WARPS), 32 * TRS_WARPS, trs_smem, s>>>(
+        (const cplx<T>*)h->tdl, (const cplx<T>*)h->tdinv, (const cplx<T>*)h->tdu,
+        (const cplx<T>*)h->tdu2, h->tpiv, bsrc, B[1], cx, x, nx, ny, n1);
+  }
+  rci_note_launch();
+  RCI_CUDA_TRY(cudaGetLastError());
 #undef RCI_SMAX_DISPATCH
   return cudaSuccess;
 }

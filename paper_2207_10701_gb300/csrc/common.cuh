@@ -78,8 +78,11 @@ static inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // in all threads and before it reads or writes anything: it waits until the kernel before has completed
 // with its writes visible (and so, in turn, everything before that), then lets its own dependent be
 // placed.  New FP64 designs: 50 x 128 6.11 -> 5.40 ms, 500 x 160 39.0 -> 38.0.
-// The FP32 kernels are launched ordinarily: alone they gained under 1 %, and with four evaluations in
-// flight their waiting blocks kept the others off idle SMs (158 -> 152 evaluations/s at 500 x 160).
+// The FP32 kernels of blocks up to 160 rows are launched ordinarily: alone they gained under 1 %, and with
+// four evaluations in flight their waiting blocks kept the others off idle SMs (158 -> 152 evaluations/s
+// at 500 x 160).  The digit products and the Gauss-Jordan kernel that the inversion by halves shares with
+// the FP64 form are dependents there too: 20 x 176, 60 x 224 and 120 x 192 take 2.5, 1.3 and 1.5 % less
+// alone, and as much less an evaluation with four in flight (4.17, 7.49 and 7.58 ms).
 __device__ __forceinline__ void dep_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -23,11 +23,11 @@
 // bound of the FP64 FMA loop is 2^-36.  So may the accumulators of the shorter forms, by 2^-23: their
 // products are corrections, or residuals that are formed again.
 //
-// Measured, 608 products of 160^3: SG_FULL 710 us (1.17 us a product, 28 TFLOP/s of FP64 work; the
+// Measured, 608 products of 160^3: SG_FULL 723 us (1.19 us a product, 28 TFLOP/s of FP64 work; the
 // FP64 GEMM takes 28 us a product; 897 us with A in shared memory and an epilogue that the MMAs
-// wait for), SG_HALF 463 us; splitting an operand 0.25 us.  Bound by the MMAs (47 cycles each at
-// N = 64 with the copies of A, where the tensor cores need 32) and by the joining of the
-// accumulators (about a fifth).
+// wait for), SG_HALF 463 us; splitting an operand 0.27 us, a right one 0.22.  Bound by the MMAs (47
+// cycles each at N = 64 with the copies of A, where the tensor cores need 32) and by the joining of
+// the accumulators (about a fifth).
 //
 // Layout.  A split form holds, per 16 terms k and digit s, planes r, i and -r of bf16 core
 // matrices (8 rows x 8 terms, 128 bytes), so every shared-memory operand is a run of contiguous
