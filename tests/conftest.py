@@ -5,10 +5,11 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# Threads of the oracle's linear algebra sleep between calls instead of spinning on their cores: for
-# milliseconds after a call they kept the serving runtime's workers from waking up, which the
-# look-ahead test takes for a wrong admission order.  (Read when numpy is loaded.)
-os.environ.setdefault("OPENBLAS_THREAD_TIMEOUT", "4")
+# Threads of the oracle's linear algebra sleep 2^18 cycles after a call (the library's default is 2^26):
+# while they spin on their cores, the serving runtime's workers wake up milliseconds late, which the
+# look-ahead test takes for a wrong admission order.  (Much less, and the oracle itself takes twice as
+# long.  Read when numpy is loaded.)
+os.environ.setdefault("OPENBLAS_THREAD_TIMEOUT", "18")
 
 
 def pytest_configure(config):
